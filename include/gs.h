@@ -165,7 +165,8 @@ typedef struct {
   size_t ranges;         /* u32 [K*Tx*Ty][2]: [start, end) of each global tile ([0, 0) when empty) */
   size_t pair_grads;     /* float [pair_capacity][12]: per-pair gradients of gs_raster_bwd, valid
                             where the pair's bit in pair_valid is set (other pairs: zero) */
-  int32_t sort_passes;   /* 8-bit LSD passes of the pair sort over the tile bits: ceil(ceil(log2(K*Tx*Ty)) / 8) */
+  int32_t sort_passes;   /* 8-bit LSD passes of the radix pair sort over the tile bits:
+                            ceil(ceil(log2(K*Tx*Ty)) / 8) */
   int32_t tiles_x, tiles_y;
   int32_t bin_sort_launches; /* kernels one gs_bin_sort launches */
   size_t pair_valid;     /* u32 [ceil(pair_capacity / 32)]: bit (slot & 31) of word slot / 32 is set
@@ -222,10 +223,13 @@ GS_API gs_status_t gs_project(const gs_config_t* cfg, const gs_gaussians_t* gaus
  * ((k*Tx*Ty + ty*Tx + tx) << 32) | depth bits emitted in (k, g) order (equal keys keep
  * (k, g) order), plus per-tile [start, end) ranges. Each sorted pair is stored as key =
  * ((k*Tx*Ty + ty*Tx + tx) << 32) | g and value = its emission index (the slot of its
- * gradient record). Computed as: a stable onesweep radix sort of the K*N items on their
- * 32-bit depth keys, an exclusive scan of tiles emitted in that order, emission in that
- * order, and a stable onesweep radix sort of the pairs on the tile bits only. The pair count stays on the device; more than pair_capacity pairs sets
- * GS_DEVERR_PAIR_OVERFLOW and only the first pair_capacity pairs are emitted. Consumes the
+ * gradient record). Computed in one of two ways, chosen from K, N and the image size: (a) the pairs
+ * go straight to their tile's list and every list is sorted on its own by (depth bits, item), or
+ * (b, few tiles or very many Gaussians per tile) a stable onesweep radix sort of the live items on
+ * their 32-bit depth keys, an exclusive scan of tiles emitted in that order, emission in that order,
+ * and a stable onesweep radix sort of the pairs on the tile bits only. The emission indices number
+ * the items' pairs in increasing item order (a) or in depth order (b). The pair count stays on the
+ * device; more than pair_capacity pairs sets GS_DEVERR_PAIR_OVERFLOW and leaves every tile empty. Consumes the
  * state of the preceding gs_project on the same workspace (call it once per gs_project). */
 GS_API gs_status_t gs_bin_sort(const gs_config_t* cfg, void* ws, size_t ws_bytes, void* stream);
 

@@ -1,5 +1,6 @@
-// Tile binning of the projected Gaussians, after the (view, Gaussian) items have been
-// stably sorted by camera depth:
+// Tile binning of the projected Gaussians by global radix sorts (grids of fewer tiles than
+// multiprocessors; larger ones take tile_sort.cu, which shares k_tile_scan), after the
+// (view, Gaussian) items have been stably sorted by camera depth:
 //   k_sorted_counts   tiles emitted per item in depth order, per-block totals
 //   k_scan_blocks     exclusive scan of the block totals, pair count, capacity check
 //   k_item_offsets    per item (depth order): first pair index, rectangle, ids
@@ -26,8 +27,8 @@ constexpr int kEmitThreads = 256;
 
 // Tiles touched by each live item in depth order, and per-chunk totals for the scan (chunks of
 // kProjBlock items; the blocks stride over the chunks of the n_live live items). Block 0 also
-// resets what the tile scan accumulates into: the pair sort's digit histograms, the per-view
-// look-back status and the view counter.
+// resets what the tile scan accumulates into: the pair sort's digit histograms, the slabs'
+// look-back status and the slab counter.
 __global__ void __launch_bounds__(kProjBlock) k_sorted_counts(Layout L, uint8_t* __restrict__ ws) {
   pdl_begin();
   Status* st = at<Status>(ws, L.status);
@@ -35,7 +36,7 @@ __global__ void __launch_bounds__(kProjBlock) k_sorted_counts(Layout L, uint8_t*
     uint32_t* hist = at<uint32_t>(ws, L.hist);
     for (int i = threadIdx.x; i < 4 * 256; i += kProjBlock) hist[i] = 0;
     uint64_t* vlb = at<uint64_t>(ws, L.view_lb);
-    for (int i = threadIdx.x; i < L.K; i += kProjBlock) vlb[i] = 0;
+    for (int i = threadIdx.x; i < L.K * L.scan_slabs; i += kProjBlock) vlb[i] = 0;
     if (threadIdx.x == 0) st->view_ctr = 0;
   }
   const int64_t n_live = st->n_live;
@@ -175,78 +176,125 @@ __global__ void __launch_bounds__(kProjBlock) k_item_offsets(Layout L, uint8_t* 
   }
 }
 
-// One block per view (views numbered in block start order): the row-wise prefix sum of the
-// view's (Ty+1) x (Tx+1) span grid (cell (ty, tx) then holds the number of pairs of tile (ty, tx);
-// staged in shared memory when it fits, else summed in place in global memory), the view's pair
-// total, the pair offset of the view (decoupled look-back over the lower-numbered views), then
-// the exclusive scan of the per-tile pair counts over the view's tiles: ranges (clamped to the
-// pairs actually emitted; [0, 0) for an empty tile) and the digit histograms of the pair sort.
-__global__ void __launch_bounds__(kScanThreads) k_tile_scan(Layout L, uint8_t* __restrict__ ws) {
+// Per-tile pair counts, ranges and what the next stage starts from. One block per slab of kScanRows
+// tile rows of a view (slabs numbered in block start order): the row-wise prefix sums of the slab's
+// part of the view's span grids (one warp per row) are the copies' pairs of every tile, kept in
+// shared memory; the exclusive scan over the slab's tiles starts from the slab's pair offset (decoupled
+// look-back over the lower-numbered slabs). Writes the ranges (clamped to the pairs actually emitted;
+// [0, 0) for an empty tile), and for the tile-sort binning the cursors of each tile's sub-lists
+// (one per copy of the span grid) and the list of tiles with more than kTileSortShort pairs, else
+// the digit histograms of the pair sort. Bound by latency (a few dependent round trips); slabs keep
+// the serial part short: one view of 3600 tiles took 28 us in one block of 1024 threads with four
+// grid copies, 12 us with one.
+constexpr int kTileScanThreads = 256;
+
+__global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(Layout L, uint8_t* __restrict__ ws) {
   pdl_begin();
-  __shared__ uint64_t tmp[32];
+  extern __shared__ uint32_t s_count[];  // [diff_copies][kScanRows * Tx]
+  constexpr int kWarps = kTileScanThreads / 32;
+  __shared__ uint64_t s_warp[kWarps];
   __shared__ uint32_t s_hist[4 * 256];
-  __shared__ int32_t sg[kProjGridCells];
-  __shared__ uint32_t s_view;
+  __shared__ uint32_t s_slab;
   __shared__ uint64_t s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Status* st = at<Status>(ws, L.status);
-  if (threadIdx.x == 0) s_view = atomicAdd(&st->view_ctr, 1u);
-  for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_hist[i] = 0;
+  if (threadIdx.x == 0) s_slab = atomicAdd(&st->view_ctr, 1u);
+  if (!L.tile_sort)
+    for (int i = threadIdx.x; i < 4 * 256; i += kTileScanThreads) s_hist[i] = 0;
   __syncthreads();
-  const int k = static_cast<int>(s_view);
-  if (k >= L.K) return;
+  const int slab = static_cast<int>(s_slab);
+  if (slab >= L.K * L.scan_slabs) return;
+  const int k = slab / L.scan_slabs, ty0 = (slab - k * L.scan_slabs) * kScanRows;
+  const int rows = L.Ty - ty0 < kScanRows ? L.Ty - ty0 : kScanRows;
+  const int tiles = rows * L.Tx, copies = L.diff_copies;
   // after a capacity overflow the pair sort does not run: leave every tile empty
-  const uint64_t n = st->total_pairs > static_cast<uint64_t>(L.cap) ? 0 : st->num_pairs;
-  uint32_t* ranges = at<uint32_t>(ws, L.ranges);
+  const uint64_t n = st->total_pairs > static_cast<uint64_t>(L.cap) ? 0 : st->total_pairs;
   const int stride = L.Tx + 1;
-  const int cells = stride * (L.Ty + 1);
-  const bool in_smem = cells <= kProjGridCells;
-  const int64_t per_view = static_cast<int64_t>(L.Tx) * L.Ty;
-  int32_t* gg = at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(k) * cells;
-  int32_t* g = in_smem ? sg : gg;
-  if (in_smem)
-    for (int i = threadIdx.x; i < cells; i += kScanThreads) sg[i] = gg[i];
+  const int64_t cells = static_cast<int64_t>(stride) * (L.Ty + 1);
+  const int32_t* grid = at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(k) * copies * cells;
+  // (one warp per row: the copies' loads and the next 32 columns' are in flight together)
+  static_assert(kWarps == kScanRows, "one warp per tile row of the slab");
+  if (warp < rows) {
+    const int32_t* row = grid + static_cast<int64_t>(ty0 + warp) * stride;
+    uint32_t* out = s_count + warp * L.Tx;
+    int32_t carry[kTileSubLists] = {}, next[kTileSubLists];
+#pragma unroll
+    for (int c = 0; c < kTileSubLists; ++c) next[c] = c < copies && lane < L.Tx ? row[c * cells + lane] : 0;
+    for (int x = lane; x < L.Tx + lane; x += 32) {
+      int32_t v[kTileSubLists];
+#pragma unroll
+      for (int c = 0; c < kTileSubLists; ++c) {
+        v[c] = next[c];
+        next[c] = c < copies && x + 32 < L.Tx ? row[c * cells + x + 32] : 0;
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+        for (int c = 0; c < kTileSubLists; ++c) {
+          const int32_t u = __shfl_up_sync(0xffffffffu, v[c], o);
+          if (lane >= o) v[c] += u;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < kTileSubLists; ++c) {
+        if (c < copies && x < L.Tx) out[c * kScanRows * L.Tx + x] = static_cast<uint32_t>(carry[c] + v[c]);
+        carry[c] += __shfl_sync(0xffffffffu, v[c], 31);
+      }
+    }
+  }
   __syncthreads();
-  // row-wise prefix sums, and the view's total (each thread sums the rows it owns)
+  // a run of consecutive tiles per thread: its pairs, the exclusive scan of the runs, then its tiles
+  const int per = (tiles + kTileScanThreads - 1) / kTileScanThreads;
+  const int r0 = static_cast<int>(threadIdx.x) * per < tiles ? static_cast<int>(threadIdx.x) * per : tiles;
+  const int r1 = r0 + per < tiles ? r0 + per : tiles;
   uint64_t mine = 0;
-  for (int y = threadIdx.x; y < L.Ty; y += kScanThreads) {
-    int32_t acc = 0;
-    for (int x = 0; x <= L.Tx; ++x) {
-      acc += g[y * stride + x];
-      g[y * stride + x] = acc;
-      if (x < L.Tx) mine += static_cast<uint32_t>(acc);
-    }
+  for (int c = 0; c < copies; ++c)
+    for (int r = r0; r < r1; ++r) mine += s_count[c * kScanRows * L.Tx + r];
+  uint64_t incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
   }
-  uint64_t total;
-  block_inclusive_scan1024(mine, tmp, &total);
-  if (threadIdx.x < 32) {
-    const uint64_t base = lb_exclusive_warp(at<uint64_t>(ws, L.view_lb), static_cast<uint32_t>(k), total, &st->err);
-    if (threadIdx.x == 0) s_base = base;
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint64_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    before += w < warp ? s_warp[w] : 0u;
+    total += s_warp[w];
+  }
+  if (warp == 0) {
+    const uint64_t base = lb_exclusive_warp(at<uint64_t>(ws, L.view_lb), static_cast<uint32_t>(slab), total, &st->err);
+    if (lane == 0) s_base = base;
   }
   __syncthreads();
-  uint64_t carry = s_base;
-  for (int64_t base = 0; base < per_view; base += kScanThreads) {
-    const int64_t r = base + threadIdx.x;
-    uint32_t c = 0;
-    if (r < per_view) {
-      const int64_t ty = r / L.Tx, tx = r - ty * L.Tx;
-      c = static_cast<uint32_t>(g[ty * stride + tx]);
+  uint64_t start = s_base + before + incl - mine;
+  const int64_t tile0 = static_cast<int64_t>(k) * L.Tx * L.Ty + static_cast<int64_t>(ty0) * L.Tx;
+  for (int r = r0; r < r1; ++r) {
+    const int64_t tg = tile0 + r;
+    uint64_t end = start;
+    for (int c = 0; c < copies; ++c) {
+      if (L.tile_sort)
+        at<uint32_t>(ws, L.tile_cursor)[(c * L.n_tiles + tg) * kCursorStride] = static_cast<uint32_t>(end < n ? end : n);
+      end += s_count[c * kScanRows * L.Tx + r];
     }
-    uint64_t tot;
-    const uint64_t incl = block_inclusive_scan1024(c, tmp, &tot);
-    if (r < per_view) {
-      const int64_t tg = k * per_view + r;
-      const uint64_t start = c ? carry + incl - c : 0, end = c ? carry + incl : 0;
-      ranges[2 * tg] = static_cast<uint32_t>(start < n ? start : n);
-      ranges[2 * tg + 1] = static_cast<uint32_t>(end < n ? end : n);
-      if (c)
-        for (int p = 0; p < L.passes; ++p)
-          atomicAdd(&s_hist[p * 256 + ((static_cast<uint32_t>(tg) >> (8 * p)) & 0xffu)], c);
+    const bool any = end > start;
+    at<uint2>(ws, L.ranges)[tg] = make_uint2(any ? static_cast<uint32_t>(start < n ? start : n) : 0u,
+                                             any ? static_cast<uint32_t>(end < n ? end : n) : 0u);
+    if (L.tile_sort) {
+      if (end - start > static_cast<uint64_t>(kTileSortShort) && n)
+        at<uint32_t>(ws, L.long_tiles)[atomicAdd(&st->n_long, 1u)] = static_cast<uint32_t>(tg);
+    } else if (any) {
+      for (int p = 0; p < L.passes; ++p)
+        atomicAdd(&s_hist[p * 256 + ((static_cast<uint32_t>(tg) >> (8 * p)) & 0xffu)], static_cast<uint32_t>(end - start));
     }
-    carry += tot;
+    start = end;
   }
+  if (L.tile_sort) return;
   __syncthreads();
   uint32_t* hist = at<uint32_t>(ws, L.hist);
-  for (int i = threadIdx.x; i < L.passes * 256; i += kScanThreads)
+  for (int i = threadIdx.x; i < L.passes * 256; i += kTileScanThreads)
     if (s_hist[i]) atomicAdd(&hist[i], s_hist[i]);
 }
 
@@ -390,6 +438,17 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit_pairs(Layout L, uint8_t* 
 
 }  // namespace
 
+cudaError_t launch_tile_scan(const Layout& L, void* ws, cudaStream_t s) {
+  const size_t smem = static_cast<size_t>(L.diff_copies) * kScanRows * L.Tx * 4;  // <= 128 KB (Tx <= 1024)
+  if (smem > 32 * 1024) {  // (images wider than 4096 pixels)
+    const cudaError_t e = cudaFuncSetAttribute(k_tile_scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kTileSubLists * kScanRows * 1024 * 4);
+    if (e != cudaSuccess) return e;
+  }
+  launch(k_tile_scan, static_cast<unsigned>(L.K * L.scan_slabs), kTileScanThreads, smem, s, L, static_cast<uint8_t*>(ws));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_bin(const Layout& L, void* ws, cudaStream_t s) {
   auto* w = static_cast<uint8_t*>(ws);
   // the live items are counted on the device: the per-item kernels stride over their chunks
@@ -398,7 +457,7 @@ cudaError_t launch_bin(const Layout& L, void* ws, cudaStream_t s) {
   launch(k_sorted_counts, item_grid, kProjBlock, 0, s, L, w);
   launch(k_scan_blocks, 1, kScanThreads, 0, s, L, w);
   launch(k_item_offsets, item_grid, kProjBlock, 0, s, L, w);
-  launch(k_tile_scan, static_cast<unsigned>(L.K), kScanThreads, 0, s, L, w);
+  launch_tile_scan(L, ws, s);
   // the emission's blocks stride over the windows of emitted pairs (their number is on the device);
   // enough blocks that a typical count takes one window per block (a block looping over several
   // windows serialises their latency-bound searches), few enough that surplus blocks cost little

@@ -25,6 +25,15 @@ constexpr int kSortTileKeys = kSortThreads * kSortItems;
 constexpr int kMaxSortPasses = 8;
 constexpr int kPairGradStride = 12;   // floats per pair gradient record (10 used)
 constexpr int kPoseBlock = 256;       // Gaussians / live items per projection-backward block
+// Tile-sort binning (tile_sort.cu): each tile's list sorted by its own block.
+constexpr int kTileSortMinTiles = 152;  // fewer tiles than SMs: the global radix sorts instead
+constexpr int kScanRows = 8;            // tile rows per block of the tile scan
+constexpr int kTileSubLists = 4;        // cursors per tile: projection block b emits into sub-list b % 4
+constexpr int kCursorStride = 8;        // u32 between two cursors: one 32-byte sector each
+constexpr int kTileSortMaxDensity = 1024;  // Gaussians per tile of a view (see make_layout)
+constexpr int64_t kTileSortMaxItems = 1 << 25;  // most Gaussians (so list entries; 27-bit bucket numbers)
+constexpr int kTileSortShort = 2048;    // longest list sorted by a short-list block
+constexpr int kTileSortGroupItems = 6400000;  // (view, Gaussian) items per emission / sort launch
 constexpr uint32_t kSpinLimit = 1u << 21;  // bounded decoupled look-back (about a second of polling)
 constexpr int kDefaultFwdPx = 2;      // pixels per thread of the compositing kernels when
 constexpr int kDefaultBwdPx = 2;      // gs_config_t leaves the choice to the library
@@ -40,9 +49,10 @@ struct Status {
   uint32_t row_ctr;         // entries of the row-span table handed out by the projection
   uint32_t loss_ctr;        // blocks of the loss-fused forward done (reset by the last one)
   uint32_t n_live;          // live items: (view, Gaussian) items that emit at least one pair
-  uint32_t view_ctr;        // tile-scan blocks started (one per view)
+  uint32_t view_ctr;        // tile-scan blocks started
   uint32_t proj_done;       // projection blocks finished (the last one scans their live counts)
   uint32_t grad_chunk_ctr;  // chunks of live items taken by the backward projection's blocks
+  uint32_t n_long;          // tiles whose list is longer than kTileSortShort (tile-sort binning)
 };
 static_assert(sizeof(Status) <= 256, "status block");
 
@@ -78,22 +88,23 @@ struct Layout {
   // table entries (int4: first entry, number of entries, -, -), its (view, Gaussian id)
   size_t item_offsets, item_rect, item_kg;
   // row-span table: per live item, its rows from the first to the last non-empty one, each an
-  // int2 (pairs of the item in earlier rows, first column | row << 16); proj_rows: per live item
-  // (first entry, number of entries). Entries are handed out by an atomic counter; at most
-  // pair_capacity of them (more is reported as a pair overflow).
-  size_t row_table, proj_rows;
+  // int2 (pairs of the item in earlier rows, first column | row << 16). Entries are handed out by
+  // an atomic counter; at most pair_capacity of them (more is reported as a pair overflow).
+  size_t row_table;
   // one bit per pair slot: set by gs_raster_bwd for every record it writes (pairs in front of
   // every pixel's last contributor of their tile); the other records are never written, their
   // gradient is zero. Cleared by the emission.
   size_t pair_valid;
   size_t tile_loss;         // float [n_tiles]: per-tile loss partials of the loss-fused forward
   // per view a (Ty+1) x (Tx+1) grid: +1 / -1 at the first / one-past-last tile of every
-  // emitted row span; its row-wise prefix sum is the number of pairs of each tile
+  // emitted row span; its row-wise prefix sum is the number of pairs of each tile (diff_copies
+  // grids per view: projection block b adds to copy b % diff_copies)
   size_t tile_diff;
+  int diff_copies;          // kTileSubLists with the tile-sort binning, else 1
   int64_t n_emit_blocks;    // ceil(cap / kEmitPairs)
   size_t emit_first, emit_last;  // u32 [n_emit_blocks]: items holding each emission block's first / last pair
   // Live items (those that emit at least one pair) and their compaction. Only live items get
-  // projection records (proj_uv, proj_conic, proj_tiles, proj_depth_key, proj_radius, proj_rows);
+  // projection records (proj_uv, proj_conic, proj_tiles, proj_depth_key, proj_radius);
   // the others are marked dead and nothing reads their records. A live item's position among
   // the live items (in increasing k N + g order) is its rank in live_mask: live_wpre[i / 32] +
   // the set bits of word i / 32 below bit i & 31 (live_rank).
@@ -105,10 +116,30 @@ struct Layout {
   //   live_off   u32 [KN]: their first pair index (emission order), clamped to the capacity
   //   live_blocks, live_bases  u32 [n_proj_groups]: live items of each projection block, and
   //              the block's first position among all live items (scanned by the last block)
-  //   view_lb    u64 [K]: look-back status of the per-view pair totals (tile scan)
+  //   view_lb    u64 [K * scan_slabs]: look-back status of the tile scan's blocks
   //   item_partials float [KN][16]: the projection backward's per-live-item partial gradients
   size_t live_mask, live_wpre, live_kg, live_count, live_rows, live_off, live_blocks, live_bases, view_lb,
       item_partials;
+  // Tile-sort binning (tile_sort = true): the pairs go straight to their tile's list (atomic
+  // cursors) and every list is sorted by (depth, item) on its own; the buffers of the item
+  // depth sort, the row-span table and the second key / value buffers are then not allocated.
+  //   stage_ell   float4 [KN][2]: ellipse of each live item, in its projection block's segment
+  //   stage_meta  uint4 [KN]: its depth key, item id, rectangle x0|x1<<16, y0|y1<<16
+  //   (its tiles emitted: sorted_counts)
+  //   block_pairs u32 [n_proj_groups], super_pairs u64, super_live u32 [ceil(n_proj_groups / 256)]:
+  //              pairs of each projection block's live items; pairs and live items of 256 blocks
+  //   tile_cursor u32 [kTileSubLists][n_tiles][kCursorStride]: next free pair of each tile's
+  //              sub-lists (entry 0)
+  //   long_tiles  u32 [n_tiles]: the tiles with lists longer than kTileSortShort
+  // The unsorted lists are uint4 (depth bits, slot, Gaussian id, -) in the first 16 pair_capacity
+  // bytes of pair_grads, which holds nothing before the backward; the rest of it is scratch of
+  // the longest lists' sorts.
+  bool tile_sort;
+  int sort_groups;          // launches the views are split over (emission, sort)
+  int sorted;               // buffer (keys[], vals[]) holding the sorted pairs
+  size_t zero_bytes;        // the buffers from `status` on that start at zero, cleared together
+  int scan_slabs;           // blocks per view of the tile scan (kScanRows tile rows each)
+  size_t stage_ell, stage_meta, block_pairs, super_pairs, super_live, tile_cursor, long_tiles;
   size_t total;
 };
 
@@ -194,6 +225,28 @@ __device__ __forceinline__ bool item_live(const uint32_t* live_mask, int64_t kg)
 // Position of live item kg among the live items.
 __device__ __forceinline__ uint32_t live_rank(const uint32_t* live_mask, const uint32_t* live_wpre, int64_t kg) {
   return live_wpre[kg >> 5] + __popc(live_mask[kg >> 5] & ((1u << (kg & 31)) - 1u));
+}
+
+// The lanes of a warp hold consecutive numbers, lane l the numbers [st, next lane's st) (none when !any).
+// Returns, for the number r0 + lane, the rank of its owner among the lanes with any (0, 1, ...); r0 and
+// the lanes' numbers cover the asked ones. One warp-wide OR and a ballot instead of a binary search
+// by shuffles (five dependent ones).
+__device__ __forceinline__ int warp_owner_rank(int st, bool any, int r0) {
+  const int local = st - r0;
+  const uint32_t heads = __reduce_or_sync(0xffffffffu, (any && local > 0 && local < 32) ? 1u << local : 0u);
+  const int before = __popc(__ballot_sync(0xffffffffu, any && local <= 0));
+  return before - 1 + __popc(heads & (0xffffffffu >> (31 - (threadIdx.x & 31))));
+}
+__device__ __forceinline__ int warp_exclusive_scan(int x, int& total) {
+  const int lane = threadIdx.x & 31;
+  int incl = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  total = __shfl_sync(0xffffffffu, incl, 31);
+  return incl - x;
 }
 
 bool make_layout(const gs_config_t* cfg, Layout* L);
@@ -335,9 +388,38 @@ __device__ __forceinline__ int2 row_span(const Ellipse& E, int ty, int x0, int x
   return make_int2(static_cast<int>(fa), static_cast<int>(fb));
 }
 
+__device__ __forceinline__ Ellipse shfl_ellipse(const Ellipse& E, int o) {
+  Ellipse e;
+  e.u = __shfl_sync(0xffffffffu, E.u, o);
+  e.v = __shfl_sync(0xffffffffu, E.v, o);
+  e.b = __shfl_sync(0xffffffffu, E.b, o);
+  e.inv_c = __shfl_sync(0xffffffffu, E.inv_c, o);
+  e.sdet = __shfl_sync(0xffffffffu, E.sdet, o);
+  e.hx = __shfl_sync(0xffffffffu, E.hx, o);
+  e.hy = __shfl_sync(0xffffffffu, E.hy, o);
+  e.kxy = __shfl_sync(0xffffffffu, E.kxy, o);
+  return e;
+}
+
+// The rows of [y0, y1) that can hold a non-empty row_span: those whose widened strip of pixel
+// centres meets E's vertical extent, with 0.02 rows + 1e-6 (|v| + hy) of slack for the rounding of
+// row_span's own test. A NaN bound leaves its side at the rectangle's edge.
+__device__ __forceinline__ int2 ellipse_rows(const Ellipse& E, int y0, int y1) {
+  const float mgy = 0.002f * E.hy + 0.05f;
+  const float slack = 0.02f + 1e-6f * (fabsf(E.v) + E.hy);
+  const float inv_t = 1.0f / static_cast<float>(kTile);
+  const float lo = ceilf((E.v - E.hy - mgy - (static_cast<float>(kTile) - 0.5f)) * inv_t - slack);
+  const float hi = floorf((E.v + E.hy + mgy - 0.5f) * inv_t + slack);
+  const int a = static_cast<int>(fmaxf(lo, static_cast<float>(y0)));
+  const int b = static_cast<int>(fminf(hi, static_cast<float>(y1 - 1))) + 1;
+  return make_int2(a, b > a ? b : a);
+}
+
 // Launchers (each defined in its own translation unit). All return cudaGetLastError().
 cudaError_t launch_project(const Layout& L, const GaussPtrs& g, const gs_camera_t* cams, void* ws, cudaStream_t s);
 cudaError_t launch_bin(const Layout& L, void* ws, cudaStream_t s);
+cudaError_t launch_tile_scan(const Layout& L, void* ws, cudaStream_t s);
+cudaError_t launch_tile_bin(const Layout& L, void* ws, cudaStream_t s);  // the tile-sort binning
 cudaError_t launch_item_sort(const Layout& L, void* ws, cudaStream_t s);
 cudaError_t launch_sort_passes(const Layout& L, void* ws, cudaStream_t s);
 

@@ -287,7 +287,9 @@ __device__ __forceinline__ Projected project_item(const Layout& L, const GaussPt
 // live_mask, its binning record (depth key, tiles emitted, item id, row-span entries) to the
 // block's segment of the staging arrays in item order (compacted by k_live_copy), its depth
 // key's digits to the item-sort histograms. The last block to finish scans the blocks' live
-// counts into their first positions among the live items.
+// counts into their first positions among the live items. For the tile-sort binning
+// (L.tile_sort) the record holds the ellipse and rectangle instead, pass 2 and the histograms
+// are left out, and the tile scan and the emission do the rest.
 // The block of items (in item order) that launched block b takes. The n blocks of items are seen
 // as rows of Bv = ceil(n / K) blocks, one row per view (rows cut at block boundaries, so a row
 // is about one view's items; the last row may be shorter), and the launch order walks this
@@ -330,18 +332,22 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
   __shared__ int32_t s_grid[kProjGridCells];
   __shared__ uint32_t s_surv[kWords], s_spre[kWords + 1], s_live[kWords];
   __shared__ uint32_t s_wcnt[kProjThreads / 32];
-  __shared__ uint32_t s_seg;
+  __shared__ uint32_t s_wpairs[kProjThreads / 32];
+  __shared__ uint32_t s_seg, s_pairs;  // the block's live items so far and their pairs
   __shared__ int s_acc[kProjThreads / 32][3][32];  // per warp and lane: tiles, first row, last row
   __shared__ int s_carry[kProjThreads / 32][32];   // tiles of an item's rows already written
+  __shared__ uint8_t s_owner[kProjThreads / 32][32];  // the lanes whose items own rows, in order
   // the first kSpanCache row spans of each warp's round (pass 1), read again by pass 2
   __shared__ int2 s_span[kProjThreads / 32][kSpanCache];
   const int gstride = L.Tx + 1;
   const int gcells = gstride * (L.Ty + 1);
   const bool use_sgrid = gcells <= kProjGridCells;
+  const int copy = static_cast<int>(blk & (L.diff_copies - 1));  // the block's copy of the span grids
   const int k_block = static_cast<int>(first / (L.N > 0 ? L.N : 1));
-  for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads) s_hist[i] = 0;
+  if (!L.tile_sort)
+    for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads) s_hist[i] = 0;
   if (threadIdx.x < kWords) s_live[threadIdx.x] = 0;
-  if (threadIdx.x == 0) s_seg = 0;
+  if (threadIdx.x == 0) s_seg = s_pairs = 0;
 
   // ---------------- phase 1: every item --------------------------------------------
   for (int r = 0; r < kWords / (kProjThreads / 32); ++r) {
@@ -420,38 +426,6 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
   __syncthreads();
 
   // ---------------- phase 2: the survivors, kProjThreads per round ---------------------
-  auto owner = [&](int st, int r) {  // the last lane whose first row number is <= r
-    int o = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const int cand = o + step;
-      const int sc = __shfl_sync(0xffffffffu, st, cand & 31);
-      if (cand < 32 && sc <= r) o = cand;
-    }
-    return o;
-  };
-  auto owner_ellipse = [&](const Ellipse& E, int o) {
-    Ellipse e;
-    e.u = __shfl_sync(0xffffffffu, E.u, o);
-    e.v = __shfl_sync(0xffffffffu, E.v, o);
-    e.b = __shfl_sync(0xffffffffu, E.b, o);
-    e.inv_c = __shfl_sync(0xffffffffu, E.inv_c, o);
-    e.sdet = __shfl_sync(0xffffffffu, E.sdet, o);
-    e.hx = __shfl_sync(0xffffffffu, E.hx, o);
-    e.hy = __shfl_sync(0xffffffffu, E.hy, o);
-    e.kxy = __shfl_sync(0xffffffffu, E.kxy, o);
-    return e;
-  };
-  auto warp_excl_scan = [&](int x, int& total) {
-    int incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    total = __shfl_sync(0xffffffffu, incl, 31);
-    return incl - x;
-  };
   uint32_t lm;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lm));
   for (int base = 0; base < n_surv; base += kProjThreads) {
@@ -479,16 +453,22 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
     s_acc[wib][2][lane] = -1;
     __syncwarp();
     int st1 = 0;  // this lane's item's first row number in pass 1
+    int2 rows = make_int2(0, 0);  // its rows [x, y) that may hold emitted tiles
     {
       int total = 0;
-      st1 = warp_excl_scan(P.live ? P.y1 - P.y0 : 0, total);
+      if (P.live) rows = ellipse_rows(P.E, P.y0, P.y1);
+      st1 = warp_exclusive_scan(rows.y - rows.x, total);
       const int st = st1;
+      const bool any = rows.y > rows.x;
+      const uint32_t owners = __ballot_sync(0xffffffffu, any);
+      if (any) s_owner[wib][__popc(owners & lm)] = static_cast<uint8_t>(lane);
+      __syncwarp();
       for (int rb = 0; rb < total; rb += 32) {
         const int r = rb + lane;
-        const int o = owner(st, r);
-        const Ellipse eo = owner_ellipse(P.E, o);
+        const int o = s_owner[wib][warp_owner_rank(st, any, rb)];
+        const Ellipse eo = shfl_ellipse(P.E, o);
         const int ox0 = __shfl_sync(0xffffffffu, P.x0, o), ox1 = __shfl_sync(0xffffffffu, P.x1, o);
-        const int oy0 = __shfl_sync(0xffffffffu, P.y0, o), ok = __shfl_sync(0xffffffffu, kv, o);
+        const int oy0 = __shfl_sync(0xffffffffu, rows.x, o), ok = __shfl_sync(0xffffffffu, kv, o);
         const int ost = __shfl_sync(0xffffffffu, st, o);
         if (r < total) {
           const int ty = oy0 + (r - ost);
@@ -500,7 +480,7 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
             atomicMax(&s_acc[wib][2][o], ty);
             int32_t* dg = (use_sgrid && ok == k_block)
                               ? s_grid
-                              : at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(ok) * gcells;
+                              : at<int32_t>(ws, L.tile_diff) + (static_cast<int64_t>(ok) * L.diff_copies + copy) * gcells;
             atomicAdd(&dg[ty * gstride + sp.x], 1);  // row-wise prefix sum: pairs per tile
             atomicAdd(&dg[ty * gstride + sp.y + 1], -1);
           }
@@ -519,9 +499,10 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
       at<uint32_t>(ws, L.proj_depth_key)[idx] = item_key;
       at<int32_t>(ws, L.proj_radius)[idx] = P.radius;
     }
-    // row-span table entries for the item's rows first..last (one counter atomic per warp)
+    // row-span table entries for the item's rows first..last (one counter atomic per warp); the
+    // tile-sort binning computes the spans again from the staged ellipse instead
     uint2 rows_out = make_uint2(0, 0);
-    {
+    if (!L.tile_sort) {
       uint32_t incl = nrows;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -535,18 +516,20 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
       if (nrows && !fits) atomicOr(&at<Status>(ws, L.status)->err, GS_DEVERR_PAIR_OVERFLOW);
       if (is_live) rows_out = fits ? make_uint2(rbase, nrows) : make_uint2(0, 0);
       int total = 0;
-      const int st = warp_excl_scan(fits ? static_cast<int>(nrows) : 0, total);
+      const int st = warp_exclusive_scan(fits ? static_cast<int>(nrows) : 0, total);
       int2* tab = at<int2>(ws, L.row_table);
       s_carry[wib][lane] = 0;
+      const uint32_t owners = __ballot_sync(0xffffffffu, fits);
+      if (fits) s_owner[wib][__popc(owners & lm)] = static_cast<uint8_t>(lane);
       __syncwarp();
       for (int b2 = 0; b2 < total; b2 += 32) {
         const int r = b2 + lane;
-        const int o = owner(st, r);
+        const int o = s_owner[wib][warp_owner_rank(st, fits, b2)];
         const int ofirst = __shfl_sync(0xffffffffu, row_first, o);
         const uint32_t obase = __shfl_sync(0xffffffffu, rbase, o);
         const int ost = __shfl_sync(0xffffffffu, st, o);
-        // the row's index in pass 1 (the owner's rows from its rectangle's first row on)
-        const int r1 = __shfl_sync(0xffffffffu, st1, o) + (ofirst - __shfl_sync(0xffffffffu, P.y0, o)) + (r - ost);
+        // the row's index in pass 1 (the owner's rows from the first examined one on)
+        const int r1 = __shfl_sync(0xffffffffu, st1, o) + (ofirst - __shfl_sync(0xffffffffu, rows.x, o)) + (r - ost);
         const bool cached = r < total && r1 < kSpanCache;
         int2 sp = make_int2(1, 0);
         int ty = 0, len = 0;
@@ -556,7 +539,7 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
             sp = s_span[wib][r1];
           }
         } else {
-          const Ellipse eo = owner_ellipse(P.E, o);
+          const Ellipse eo = shfl_ellipse(P.E, o);
           const int ox0 = __shfl_sync(0xffffffffu, P.x0, o), ox1 = __shfl_sync(0xffffffffu, P.x1, o);
           if (r < total) {
             ty = ofirst + (r - ost);
@@ -584,25 +567,43 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
     // the live items of this round, in item order: their bits, and their binning records at
     // the end of the block's segment
     const uint32_t ballot = __ballot_sync(0xffffffffu, is_live);
-    if (lane == 0) s_wcnt[wib] = __popc(ballot);
+    const uint32_t wpairs = __reduce_add_sync(0xffffffffu, is_live ? count : 0u);
+    if (lane == 0) {
+      s_wcnt[wib] = __popc(ballot);
+      s_wpairs[wib] = wpairs;
+    }
     __syncthreads();
-    uint32_t before = s_seg;
-    for (int w = 0; w < wib; ++w) before += s_wcnt[w];
+    // (the round's totals are read between the barriers: the next round overwrites the warps' counts)
+    uint32_t before = s_seg, round_live = 0, round_pairs = 0;
+#pragma unroll
+    for (int w = 0; w < kProjThreads / 32; ++w) {
+      const uint32_t c = s_wcnt[w];
+      before += w < wib ? c : 0u;
+      round_live += c;
+      round_pairs += s_wpairs[w];
+    }
     if (is_live) {
       atomicOr(&s_live[(idx - first) >> 5], 1u << (idx & 31));
       const int64_t pos = first + before + __popc(ballot & lm);
-      at<uint32_t>(ws, L.item_keys[1])[pos] = item_key;        // staging: depth-sort key
-      at<uint32_t>(ws, L.item_vals[1])[pos] = static_cast<uint32_t>(idx);  // staging: item id
       at<uint32_t>(ws, L.sorted_counts)[pos] = count;          // staging: tiles emitted
-      at<uint2>(ws, L.item_rect)[pos] = rows_out;              // staging: row-span entries (as uint2)
+      if (L.tile_sort) {
+        const Ellipse& E = P.E;
+        at<float4>(ws, L.stage_ell)[2 * pos] = make_float4(E.u, E.v, E.b, E.inv_c);
+        at<float4>(ws, L.stage_ell)[2 * pos + 1] = make_float4(E.sdet, E.hx, E.hy, E.kxy);
+        at<uint4>(ws, L.stage_meta)[pos] =
+            make_uint4(item_key, static_cast<uint32_t>(idx), pack16(P.x0, P.x1), pack16(P.y0, P.y1));
+      } else {
+        at<uint32_t>(ws, L.item_keys[1])[pos] = item_key;        // staging: depth-sort key
+        at<uint32_t>(ws, L.item_vals[1])[pos] = static_cast<uint32_t>(idx);  // staging: item id
+        at<uint2>(ws, L.item_rect)[pos] = rows_out;              // staging: row-span entries (as uint2)
 #pragma unroll
-      for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p * 256 + ((item_key >> (8 * p)) & 0xffu)], 1u);
+        for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p * 256 + ((item_key >> (8 * p)) & 0xffu)], 1u);
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      uint32_t tot = 0;
-      for (int w = 0; w < kProjThreads / 32; ++w) tot += s_wcnt[w];
-      s_seg += tot;
+      s_seg += round_live;
+      s_pairs += round_pairs;
     }
   }
   __syncthreads();
@@ -613,9 +614,22 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
   }
   if (threadIdx.x == 0) at<uint32_t>(ws, L.live_blocks)[blk] = s_seg;
   if (use_sgrid && n_surv > 0 && k_block < L.K) {
-    int32_t* dg = at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(k_block) * gcells;
+    int32_t* dg = at<int32_t>(ws, L.tile_diff) + (static_cast<int64_t>(k_block) * L.diff_copies + copy) * gcells;
     for (int i = threadIdx.x; i < gcells; i += kProjThreads)
       if (s_grid[i]) atomicAdd(&dg[i], s_grid[i]);
+  }
+  if (L.tile_sort) {  // the emission finds the blocks' first positions; the item sort does not run
+    if (threadIdx.x == 0) {
+      at<uint32_t>(ws, L.block_pairs)[blk] = s_pairs;
+      if (s_pairs) {
+        using u64 = unsigned long long;
+        atomicAdd(reinterpret_cast<u64*>(at<uint64_t>(ws, L.super_pairs) + blk / 256), static_cast<u64>(s_pairs));
+        atomicAdd(at<uint32_t>(ws, L.super_live) + blk / 256, s_seg);
+        atomicAdd(reinterpret_cast<u64*>(&at<Status>(ws, L.status)->total_pairs), static_cast<u64>(s_pairs));
+      }
+    }
+    pdl_trigger();
+    return;
   }
   uint32_t* hist = at<uint32_t>(ws, L.item_hist);
   for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads)
@@ -712,7 +726,8 @@ cudaError_t launch_project(const Layout& L, const GaussPtrs& g, const gs_camera_
   auto* w = static_cast<uint8_t*>(ws);
   const unsigned groups = static_cast<unsigned>(L.n_proj_groups);
   launch(k_project, groups, kProjThreads, 0, s, L, g, cams, w);
-  launch(k_live_copy, groups, kProjThreads, 0, s, L, w);
+  // (the tile-sort binning's emission compacts the live items itself)
+  if (!L.tile_sort) launch(k_live_copy, groups, kProjThreads, 0, s, L, w);
   return cudaGetLastError();
 }
 

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   const TileCoord tc = tile_coord(L, blockIdx.x);
   const int lx = threadIdx.x & (kTile - 1), ly = (threadIdx.x / kTile) * PX;
   const int px = tc.tx * kTile + lx, py = tc.ty * kTile + ly;
-  const uint64_t* keys = at<uint64_t>(ws, (L.passes & 1) ? L.keys[1] : L.keys[0]);
+  const uint64_t* keys = at<uint64_t>(ws, L.sorted ? L.keys[1] : L.keys[0]);
   const uint2 rg = at<uint2>(ws, L.ranges)[blockIdx.x];
   const float ox = static_cast<float>(tc.tx * kTile), oy = static_cast<float>(tc.ty * kTile);
   const float pxc = static_cast<float>(lx) + 0.5f, pyc = static_cast<float>(ly) + 0.5f;

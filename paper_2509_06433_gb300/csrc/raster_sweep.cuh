@@ -95,8 +95,8 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
   constexpr int kWarps = kThreads / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lx = threadIdx.x & (kTile - 1), ly = (threadIdx.x / kTile) * PX;
-  const uint64_t* keys = at<uint64_t>(ws, (L.passes & 1) ? L.keys[1] : L.keys[0]);
-  const uint32_t* slots = at<uint32_t>(ws, (L.passes & 1) ? L.vals[1] : L.vals[0]);  // emission index = record slot
+  const uint64_t* keys = at<uint64_t>(ws, L.sorted ? L.keys[1] : L.keys[0]);
+  const uint32_t* slots = at<uint32_t>(ws, L.sorted ? L.vals[1] : L.vals[0]);  // emission index = record slot
   const float ox = static_cast<float>(tc.tx * kTile), oy = static_cast<float>(tc.ty * kTile);
   const float pxc = static_cast<float>(lx) + 0.5f, pyc = static_cast<float>(ly) + 0.5f;
   const uint32_t wrows = ((1u << (2 * PX)) - 1u) << ((threadIdx.x >> 5) * 2 * PX);

@@ -299,6 +299,8 @@ int device_sms() {
 cudaError_t launch_onesweep(const SortArgs& a, cudaStream_t s) { return onesweep_passes(a, s); }
 
 int bin_sort_launch_count(const Layout& L) {
+  // tile sort: the tile scan, per group of views the emission and the short lists, the long lists
+  if (L.tile_sort) return 2 + 2 * L.sort_groups;
   // counts, scan, item offsets, tile scan, emission; 4 item passes; pair passes
   return 5 + (L.KN > 0 ? 4 : 0) + L.passes;
 }

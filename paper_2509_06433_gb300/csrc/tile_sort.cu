@@ -1,0 +1,559 @@
+// Tile-sort binning: the pairs of the live items go straight to their tile's list, and every list
+// is sorted by (depth bits, item) on its own, one block per tile.
+//   k_tile_scan (binning.cu)  per-tile pair counts -> ranges, sub-lists, long tiles
+//   k_tile_emit               compaction of the live items; one unsorted record per pair
+//   k_tile_sort               lists of up to kTileSortShort pairs, in shared memory
+//   k_tile_sort_long          longer lists, cut by depth into pieces that fit in shared memory
+//
+// Order: a tile's list in (depth bits, k N + g) order, as a stable sort of ((tile << 32) | depth)
+// keys emitted in (k, g) order leaves it. A pair's slot (emission index) is its item's first pair
+// plus the pair's number in the item, the items taken in increasing k N + g order, so within a
+// tile equal depths are ordered by slot: the sort key is the 64-bit (depth bits, slot), unique, and
+// the result does not depend on the order in which the emission's atomic cursors filled the list.
+//
+// Why: the lists are short (tens to a few thousand pairs) and independent, so a tile's whole sort
+// fits in one block's shared memory: one read and one write of the pairs, where the global radix
+// sorts take four passes over the items, three scans and ceil(tile bits / 8) passes over the pairs,
+// each a dependent launch. Grids of fewer tiles than multiprocessors keep the global sorts (a block
+// per tile would leave the GPU idle and make the lists long).
+//
+// The sort of a list: one distribution pass into at most n + 256 buckets for n pairs, then each pair
+// counts the smaller keys of its own bucket. The buckets adapt to the depths' distribution: 256
+// equal slices of the list's depth range are counted first, and a slice of n pairs is cut into the
+// largest power of two <= n buckets (a wall seen next to a near object would otherwise fall into a
+// few buckets). A list that still has a bucket of more than kMaxBucket pairs (many equal or
+// almost equal depths) is sorted by a bitonic network instead.
+#include "gs_internal.cuh"
+
+namespace gs {
+namespace {
+
+constexpr int kEmitThreads = 256;
+constexpr int kShortThreads = 256;
+constexpr int kLongThreads = 512;
+constexpr int kLongBlocks = 3;    // resident per SM (75 KB of shared memory each)
+constexpr int kLongShared = 4608;  // longest list sorted in one piece
+constexpr int kLongSlices = 2048;  // depth slices a longer one is cut into
+constexpr uint32_t kMaxBucket = 64;
+constexpr int kSlices = 256;
+
+// One block per projection block: compacts its live items (in item order) and writes one record
+// (depth bits, slot, Gaussian id) per pair at the next free place of its tile's sub-list: the tile
+// scan has split every list between the projection blocks b with the same b % kTileSubLists. The
+// rate is set by the cursors' atomics, about one per 30 cycles on one address and fewer when the
+// cursors of neighbouring tiles share a 32-byte sector, so that the fullest tile decides: one sector
+// per cursor and four cursors per tile. The rows of a warp's items are numbered consecutively and examined one per lane (row_span gives the same
+// tiles as in the projection), then the pairs of those 32 rows are numbered consecutively and
+// written one per lane, four rounds in flight, so that tall or wide items do not idle the warp.
+__global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t* __restrict__ ws, int64_t block0) {
+  pdl_wait();
+  constexpr int kWarps = kEmitThreads / 32;
+  const int64_t b = block0 + blockIdx.x, first = b * L.proj_items;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  Status* st = at<Status>(ws, L.status);
+  __shared__ uint32_t s_cnt[2][kWarps], s_live[kWarps];
+  __shared__ uint64_t s_pairs[kWarps];
+  __shared__ uint32_t s_w0;
+  __shared__ uint8_t s_row[kWarps][32];
+  const uint32_t cnt = at<uint32_t>(ws, L.live_blocks)[b];
+  const uint64_t cap = static_cast<uint64_t>(L.cap), total_pairs = st->total_pairs;
+  const bool overflow = total_pairs > cap;  // every tile's range is empty
+  // the block's first live item and first pair: the sums over 256 blocks before it, then over blocks
+  uint32_t base = 0, total_live = 0;
+  uint64_t pairs = 0;
+  {
+    const int64_t super = b / 256, n_super = (L.n_proj_groups + 255) / 256;
+    for (int64_t i = threadIdx.x; i < n_super; i += kEmitThreads) {
+      const uint32_t l = at<uint32_t>(ws, L.super_live)[i];
+      total_live += l;
+      if (i < super) {
+        base += l;
+        pairs += at<uint64_t>(ws, L.super_pairs)[i];
+      }
+    }
+    const int64_t i = super * 256 + threadIdx.x;
+    static_assert(kEmitThreads == 256, "one block of the group per thread");
+    if (i < b) {
+      base += at<uint32_t>(ws, L.live_blocks)[i];
+      pairs += at<uint32_t>(ws, L.block_pairs)[i];
+    }
+    base = __reduce_add_sync(0xffffffffu, base);
+    total_live = __reduce_add_sync(0xffffffffu, total_live);
+    pairs = warp_sum_u64(pairs);
+    if (lane == 0) {
+      s_live[wib] = base;
+      s_pairs[wib] = pairs;
+      s_cnt[1][wib] = total_live;
+    }
+    __syncthreads();
+    base = 0, pairs = 0, total_live = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      base += s_live[w];
+      pairs += s_pairs[w];
+      total_live += s_cnt[1][w];
+    }
+  }
+  if (b == 0 && threadIdx.x == 0) {
+    st->n_live = total_live;
+    st->num_pairs = static_cast<uint32_t>(overflow ? cap : total_pairs);
+    if (overflow) atomicOr(&st->err, GS_DEVERR_PAIR_OVERFLOW);
+  }
+  // the record bits of the backward pass: this block's share
+  {
+    const int64_t words = (static_cast<int64_t>(overflow ? cap : total_pairs) + 31) / 32;
+    uint32_t* valid = at<uint32_t>(ws, L.pair_valid);
+    for (int64_t i = words * b / L.n_proj_groups + threadIdx.x; i < words * (b + 1) / L.n_proj_groups; i += kEmitThreads)
+      valid[i] = 0;
+  }
+  // rank bases of the block's live-mask words (warps 0-1: up to 64 words)
+  if (threadIdx.x < 64) {
+    const int64_t w = first / 32 + threadIdx.x;
+    const bool in = threadIdx.x < L.proj_items / 32 && w < (L.KN + 31) / 32;
+    const uint32_t c = in ? __popc(at<uint32_t>(ws, L.live_mask)[w]) : 0u;
+    int total;
+    const uint32_t excl = static_cast<uint32_t>(warp_exclusive_scan(static_cast<int>(c), total));
+    if (threadIdx.x == 0) s_w0 = static_cast<uint32_t>(total);
+    asm volatile("bar.sync 1, 64;" ::: "memory");  // the two warps of the mask words
+    if (in) at<uint32_t>(ws, L.live_wpre)[w] = base + excl + (threadIdx.x >= 32 ? s_w0 : 0u);
+  }
+  const int64_t per_view = static_cast<int64_t>(L.Tx) * L.Ty;
+  uint32_t* cursor = at<uint32_t>(ws, L.tile_cursor) + (b & (kTileSubLists - 1)) * L.n_tiles * kCursorStride;
+  uint4* rec = at<uint4>(ws, L.pair_grads);
+  int buf = 0;  // (s_cnt[1] is read before the first round's barrier, written after it)
+  for (uint32_t j0 = 0; j0 < cnt; j0 += kEmitThreads, buf ^= 1) {
+    // an equal share of the round's items for every warp
+    const uint32_t share = (min(cnt - j0, static_cast<uint32_t>(kEmitThreads)) + kWarps - 1) / kWarps;
+    const uint32_t j = j0 + wib * share + lane;
+    const bool valid = lane < static_cast<int>(share) && j < cnt;
+    Ellipse E{};
+    uint4 meta = make_uint4(0, 0, 0, 0);
+    uint32_t n = 0;
+    if (valid) {
+      const float4 a = at<float4>(ws, L.stage_ell)[2 * (first + j)], c = at<float4>(ws, L.stage_ell)[2 * (first + j) + 1];
+      E = Ellipse{a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+      meta = at<uint4>(ws, L.stage_meta)[first + j];
+      n = at<uint32_t>(ws, L.sorted_counts)[first + j];
+    }
+    int wtotal;
+    const uint32_t excl = static_cast<uint32_t>(warp_exclusive_scan(static_cast<int>(n), wtotal));
+    if (lane == 0) s_cnt[buf][wib] = static_cast<uint32_t>(wtotal);
+    __syncthreads();
+    uint64_t wbase = pairs;  // the warp's first pair
+    for (int w = 0; w < kWarps; ++w) {
+      wbase += w < wib ? s_cnt[buf][w] : 0u;
+      pairs += s_cnt[buf][w];
+    }
+    uint32_t g = 0, tile0 = 0;
+    if (valid) {
+      const uint64_t off = wbase + excl;
+      at<uint32_t>(ws, L.live_kg)[base + j] = meta.y;
+      at<uint32_t>(ws, L.live_count)[base + j] = n;
+      at<uint32_t>(ws, L.live_off)[base + j] = static_cast<uint32_t>(off < cap ? off : cap);
+      const uint32_t k = meta.y / static_cast<uint32_t>(L.N);
+      g = meta.y - k * static_cast<uint32_t>(L.N);
+      tile0 = static_cast<uint32_t>(k * per_view);
+    }
+    if (overflow) continue;
+    const int x0 = static_cast<int>(meta.z & 0xffffu), x1 = static_cast<int>(meta.z >> 16);
+    int2 rows = make_int2(0, 0);
+    if (valid) rows = ellipse_rows(E, static_cast<int>(meta.w & 0xffffu), static_cast<int>(meta.w >> 16));
+    int nrows;
+    const int rst = warp_exclusive_scan(rows.y - rows.x, nrows);
+    // (the lanes holding an item come first and every one of them has rows, so the rank is the lane)
+    const bool any_rows = rows.y > rows.x;
+    uint32_t slot0 = static_cast<uint32_t>(wbase);  // first pair of the next 32 rows (total <= cap < 2^30)
+    for (int rb = 0; rb < nrows; rb += 32) {
+      const int r = rb + lane;
+      const int o = warp_owner_rank(rst, any_rows, rb);
+      const Ellipse eo = shfl_ellipse(E, o);
+      const int ox0 = __shfl_sync(0xffffffffu, x0, o), ox1 = __shfl_sync(0xffffffffu, x1, o);
+      const int ty = __shfl_sync(0xffffffffu, rows.x, o) + (r - __shfl_sync(0xffffffffu, rst, o));
+      const uint32_t row_depth = __shfl_sync(0xffffffffu, meta.x, o), row_g = __shfl_sync(0xffffffffu, g, o);
+      const uint32_t row_tile0 = __shfl_sync(0xffffffffu, tile0, o);
+      int len = 0;
+      uint32_t tile = 0;
+      if (r < nrows) {
+        const int2 sp = row_span(eo, ty, ox0, ox1);
+        len = sp.x <= sp.y ? sp.y - sp.x + 1 : 0;
+        tile = row_tile0 + static_cast<uint32_t>(ty * L.Tx + sp.x);
+      }
+      int total;
+      const int pst = warp_exclusive_scan(len, total);
+      // the rows with tiles, in order (all of them but for gaps between tiles' pixel centres)
+      const uint32_t full = __ballot_sync(0xffffffffu, len > 0);
+      if (len > 0) s_row[wib][__popc(full & ((1u << lane) - 1u))] = static_cast<uint8_t>(lane);
+      __syncwarp();
+      for (int pb = 0; pb < total; pb += 128) {
+        uint32_t pos[4], dep[4], gid[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int p = pb + 32 * q + lane;
+          pos[q] = 0xffffffffu;
+          if (pb + 32 * q >= total) continue;  // (warp-uniform)
+          const int ro = s_row[wib][warp_owner_rank(pst, len > 0, pb + 32 * q)];
+          const size_t t = __shfl_sync(0xffffffffu, tile, ro) + static_cast<uint32_t>(p - __shfl_sync(0xffffffffu, pst, ro));
+          dep[q] = __shfl_sync(0xffffffffu, row_depth, ro);
+          gid[q] = __shfl_sync(0xffffffffu, row_g, ro);
+          if (p < total && GS_INDEX_OK(t < static_cast<uint64_t>(L.n_tiles), &st->err))
+            pos[q] = atomicAdd(&cursor[t * kCursorStride], 1u);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (pos[q] == 0xffffffffu) continue;
+          if (!GS_INDEX_OK(pos[q] < cap, &st->err)) continue;
+          rec[pos[q]] = make_uint4(dep[q], slot0 + static_cast<uint32_t>(pb + 32 * q + lane), gid[q], 0u);
+        }
+      }
+      slot0 += static_cast<uint32_t>(total);
+      __syncwarp();  // s_row is read before the next 32 rows overwrite it
+    }
+  }
+  pdl_trigger();
+}
+
+// Working arrays of one list's sort, in shared memory or (GLOBAL) in the list's share of scratch:
+// keys, their Gaussian ids (first the depths), the buckets' counts / ends.
+template <bool GLOBAL>
+struct SortArrays {
+  uint64_t* key;
+  uint32_t* gid;
+  uint32_t* fine;  // one word per bucket (GLOBAL) or two 16-bit buckets per word
+};
+// Words of the bucket counts of n pairs: at most n + kSlices buckets.
+template <bool GLOBAL>
+__host__ __device__ constexpr uint32_t bucket_words(uint32_t n) {
+  return GLOBAL ? n + kSlices : (n + kSlices + 1) / 2;
+}
+struct SortShared {
+  uint32_t slice[kSlices];     // pairs of each slice, then its first bucket << 5 | bucket bits
+  uint32_t warp[3][32];
+  uint32_t n_fine, max_bucket;
+};
+
+// One more pair in bucket f; returns the bucket's count before.
+template <bool GLOBAL>
+__device__ __forceinline__ uint32_t bucket_add(uint32_t* fine, uint32_t f) {
+  if (GLOBAL) return atomicAdd(&fine[f], 1u);
+  const uint32_t sh = 16 * (f & 1u);
+  return (atomicAdd(&fine[f >> 1], 1u << sh) >> sh) & 0xffffu;
+}
+template <bool GLOBAL>
+__device__ __forceinline__ uint32_t bucket_get(const uint32_t* fine, uint32_t f) {
+  if (GLOBAL) return __ldcg(&fine[f]);  // (global counts are changed by atomics, which pass the L1 by)
+  return reinterpret_cast<const uint16_t*>(fine)[f];
+}
+
+// Exclusive prefix of x over the block's threads; *total: the block's sum. tmp: 32 words, not
+// written by anyone else before the next barrier.
+template <int THREADS>
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* tmp, uint32_t* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int wtotal;
+  const uint32_t excl = static_cast<uint32_t>(warp_exclusive_scan(static_cast<int>(x), wtotal));
+  if (lane == 0) tmp[warp] = static_cast<uint32_t>(wtotal);
+  __syncthreads();
+  uint32_t before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < THREADS / 32; ++w) {
+    const uint32_t c = tmp[w];
+    before += w < warp ? c : 0u;
+    all += c;
+  }
+  *total = all;
+  return before + excl;
+}
+
+// Sorts the n records rec[0, n) of tile `tile`; writes keys_out[i] = (tile << 32) | Gaussian id and
+// vals_out[i] = slot. All threads of the block call it.
+template <int THREADS, bool GLOBAL>
+__device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_t n, SortArrays<GLOBAL> A, SortShared& S,
+                                          uint64_t tile, uint64_t* __restrict__ keys_out,
+                                          uint32_t* __restrict__ vals_out) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // the depths and their range
+  uint32_t lo = 0xffffffffu, hi = 0;
+  for (uint32_t i = t; i < n; i += THREADS) {
+    const uint32_t d = rec[i].x;
+    A.gid[i] = d;
+    lo = min(lo, d);
+    hi = max(hi, d);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    S.warp[0][warp] = lo;
+    S.warp[1][warp] = hi;
+  }
+  if (t < kSlices) S.slice[t] = 0;
+  if (t == 0) S.max_bucket = 0;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < THREADS / 32; ++w) {
+    lo = min(lo, S.warp[0][w]);
+    hi = max(hi, S.warp[1][w]);
+  }
+  const int bits = 32 - __clz(hi - lo), shift = bits > 8 ? bits - 8 : 0;
+  // pairs per slice, buckets per slice
+  for (uint32_t i = t; i < n; i += THREADS) atomicAdd(&S.slice[(A.gid[i] - lo) >> shift], 1u);
+  __syncthreads();
+  uint32_t fbits = 0, nf = 0;
+  if (t < kSlices) {
+    const uint32_t c = S.slice[t];
+    fbits = c > 1 ? min(shift, 31 - __clz(c)) : 0;
+    nf = 1u << fbits;
+  }
+  uint32_t n_fine;
+  const uint32_t f0 = block_scan<THREADS>(nf, S.warp[2], &n_fine);
+  if (t < kSlices) S.slice[t] = (f0 << 5) | fbits;
+  const uint32_t words = GLOBAL ? n_fine : (n_fine + 1) / 2;
+  for (uint32_t i = t; i < words; i += THREADS) A.fine[i] = 0;
+  __syncthreads();
+  const uint32_t rest = (1u << shift) - 1u;  // (shift <= 24)
+  auto bucket = [&](uint32_t d) {
+    const uint32_t s = S.slice[(d - lo) >> shift];
+    return (s >> 5) + (((d - lo) & rest) >> (shift - (s & 31u)));
+  };
+  for (uint32_t i = t; i < n; i += THREADS) bucket_add<GLOBAL>(A.fine, bucket(A.gid[i]));
+  __syncthreads();
+  // exclusive prefix of the bucket counts (a run of consecutive words per thread)
+  {
+    const uint32_t per = ((words + THREADS - 1) / THREADS) | 1u;  // odd: the runs start in different banks
+    const uint32_t i0 = min(t * per, words), i1 = min(i0 + per, words);
+    uint32_t sum = 0, most = 0;
+    for (uint32_t i = i0; i < i1; ++i) {
+      const uint32_t c = GLOBAL ? __ldcg(&A.fine[i]) : A.fine[i];
+      const uint32_t c0 = GLOBAL ? c : c & 0xffffu, c1 = GLOBAL ? 0u : c >> 16;
+      sum += c0 + c1;
+      most = max(most, max(c0, c1));
+    }
+    uint32_t all;
+    uint32_t at0 = block_scan<THREADS>(sum, S.warp[0], &all);
+    for (uint32_t i = i0; i < i1; ++i) {
+      const uint32_t c = GLOBAL ? __ldcg(&A.fine[i]) : A.fine[i];
+      const uint32_t c0 = GLOBAL ? c : c & 0xffffu, c1 = GLOBAL ? 0u : c >> 16;
+      A.fine[i] = GLOBAL ? at0 : (at0 | ((at0 + c0) << 16));
+      at0 += c0 + c1;
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0 && most > kMaxBucket) S.max_bucket = most;  // (any of them: only whether there is one)
+  }
+  __syncthreads();
+  // into the buckets; afterwards fine[f] is bucket f's end
+  for (uint32_t i = t; i < n; i += THREADS) {
+    const uint4 r = rec[i];
+    const uint32_t pos = bucket_add<GLOBAL>(A.fine, bucket(r.x));
+    A.key[pos] = (static_cast<uint64_t>(r.x) << 32) | r.y;
+    A.gid[pos] = r.z;
+  }
+  __syncthreads();
+  const uint64_t hi_word = tile << 32;
+  if (S.max_bucket == 0) {
+    for (uint32_t i = t; i < n; i += THREADS) {
+      const uint64_t key = A.key[i];
+      const uint32_t f = bucket(static_cast<uint32_t>(key >> 32));
+      const uint32_t s = f ? bucket_get<GLOBAL>(A.fine, f - 1) : 0u, e = bucket_get<GLOBAL>(A.fine, f);
+      uint32_t rank = s;
+      for (uint32_t j = s; j < e; ++j) rank += A.key[j] < key ? 1u : 0u;
+      keys_out[rank] = hi_word | A.gid[i];
+      vals_out[rank] = static_cast<uint32_t>(key);
+    }
+    return;
+  }
+  // bitonic network over the next power of two (absent keys compare as the largest)
+  uint32_t m = 1;
+  while (m < n) m <<= 1;
+  for (uint32_t k = 2; k <= m; k <<= 1) {
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      for (uint32_t q = t; q < m / 2; q += THREADS) {
+        // the first step of a merge compares mirrored positions, so every comparison is ascending
+        const uint32_t a = (q / j) * 2 * j + (q % j);
+        const uint32_t c = (j == k >> 1) ? (q / j) * 2 * j + (2 * j - 1 - q % j) : a + j;
+        if (c < n) {
+          const uint64_t ka = A.key[a], kc = A.key[c];
+          if (kc < ka) {
+            A.key[a] = kc;
+            A.key[c] = ka;
+            const uint32_t ga = A.gid[a];
+            A.gid[a] = A.gid[c];
+            A.gid[c] = ga;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (uint32_t i = t; i < n; i += THREADS) {
+    keys_out[i] = hi_word | A.gid[i];
+    vals_out[i] = static_cast<uint32_t>(A.key[i]);
+  }
+}
+
+template <int CAP>
+struct ListSmem {
+  uint64_t key[CAP];
+  uint32_t gid[CAP];
+  uint32_t fine[bucket_words<false>(CAP)];
+  SortShared S;
+};
+
+__global__ void __launch_bounds__(kShortThreads) k_tile_sort(Layout L, uint8_t* __restrict__ ws, int64_t tile0) {
+  pdl_wait();
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  ListSmem<kTileSortShort>& M = *reinterpret_cast<ListSmem<kTileSortShort>*>(smem_raw);
+  const int64_t tile = tile0 + blockIdx.x;
+  const uint2 rg = at<uint2>(ws, L.ranges)[tile];
+  const uint32_t n = rg.y - rg.x;
+  if (n > 0 && n <= static_cast<uint32_t>(kTileSortShort))
+    sort_list<kShortThreads, false>(at<uint4>(ws, L.pair_grads) + rg.x, n, SortArrays<false>{M.key, M.gid, M.fine}, M.S,
+                                    static_cast<uint64_t>(tile), at<uint64_t>(ws, L.keys[0]) + rg.x,
+                                    at<uint32_t>(ws, L.vals[0]) + rg.x);
+  pdl_trigger();
+}
+
+// The lists longer than kTileSortShort, taken from the tile scan's list by a grid of resident blocks.
+// A list of more than kLongShared pairs is first cut by depth: its records go, in the order of
+// kLongSlices equal slices of its depth range, to the list's share of scratch, and runs of slices that
+// fit are sorted in shared memory one after another (a single slice that does not fit is sorted in
+// global memory). Behind the unsorted records, a list that starts at pair s owns the 32 bytes per
+// pair of pair_grads from byte 16 capacity + 32 s on: 16 n bytes of cut records, then the buckets of
+// a global sort, whose keys and ids take the place of the unsorted records.
+struct LongSmem {
+  ListSmem<kLongShared> list;
+  uint32_t slice[kLongSlices];
+  uint32_t lo[kLongThreads / 32], hi[kLongThreads / 32];
+};
+
+__global__ void __launch_bounds__(kLongThreads, kLongBlocks) k_tile_sort_long(Layout L, uint8_t* __restrict__ ws) {
+  pdl_wait();
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  LongSmem& M = *reinterpret_cast<LongSmem*>(smem_raw);
+  const SortArrays<false> shared{M.list.key, M.list.gid, M.list.fine};
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t n_long = at<Status>(ws, L.status)->n_long;
+  for (uint32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
+    const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[i];
+    const uint2 rg = at<uint2>(ws, L.ranges)[tile];
+    const uint32_t n = rg.y - rg.x;
+    uint4* rec = at<uint4>(ws, L.pair_grads) + rg.x;
+    uint64_t* keys = at<uint64_t>(ws, L.keys[0]) + rg.x;
+    uint32_t* vals = at<uint32_t>(ws, L.vals[0]) + rg.x;
+    if (n <= static_cast<uint32_t>(kLongShared)) {
+      sort_list<kLongThreads, false>(rec, n, shared, M.list.S, tile, keys, vals);
+      __syncthreads();  // the next list reuses the shared arrays
+      continue;
+    }
+    uint8_t* scratch = ws + L.pair_grads + 16 * static_cast<size_t>(L.cap) + 32 * static_cast<size_t>(rg.x);
+    uint4* cut = reinterpret_cast<uint4*>(scratch);
+    uint32_t lo = 0xffffffffu, hi = 0;
+    for (uint32_t j = t; j < n; j += kLongThreads) {
+      const uint32_t d = rec[j].x;
+      lo = min(lo, d);
+      hi = max(hi, d);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      M.lo[warp] = lo;
+      M.hi[warp] = hi;
+    }
+    for (int s = t; s < kLongSlices; s += kLongThreads) M.slice[s] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kLongThreads / 32; ++w) {
+      lo = min(lo, M.lo[w]);
+      hi = max(hi, M.hi[w]);
+    }
+    constexpr int kBits = 11;
+    static_assert(kLongSlices == 1 << kBits, "slices of a power-of-two width");
+    const int bits = 32 - __clz(hi - lo), shift = bits > kBits ? bits - kBits : 0;
+    for (uint32_t j = t; j < n; j += kLongThreads) atomicAdd(&M.slice[(rec[j].x - lo) >> shift], 1u);
+    __syncthreads();
+    {
+      constexpr int kPer = kLongSlices / kLongThreads;
+      uint32_t c[kPer], sum = 0, all;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        c[q] = M.slice[t * kPer + q];
+        sum += c[q];
+      }
+      uint32_t at0 = block_scan<kLongThreads>(sum, M.list.S.warp[0], &all);
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        M.slice[t * kPer + q] = at0;
+        at0 += c[q];
+      }
+    }
+    __syncthreads();
+    for (uint32_t j = t; j < n; j += kLongThreads) {
+      const uint4 r = rec[j];
+      cut[atomicAdd(&M.slice[(r.x - lo) >> shift], 1u)] = r;
+    }
+    __syncthreads();  // slice[s] is now slice s's end
+    uint32_t start = 0;
+    for (int s0 = 0; s0 < kLongSlices && start < n;) {
+      int a = s0, b = kLongSlices;  // the most slices [s0, a) whose records fit
+      while (a < b) {
+        const int mid = (a + b + 1) / 2;
+        if (M.slice[mid - 1] - start <= static_cast<uint32_t>(kLongShared)) a = mid; else b = mid - 1;
+      }
+      if (a > s0) {
+        const uint32_t m = M.slice[a - 1] - start;
+        if (m > 0) sort_list<kLongThreads, false>(cut + start, m, shared, M.list.S, tile, keys + start, vals + start);
+        start += m;
+        s0 = a;
+      } else {
+        const uint32_t m = M.slice[s0] - start;
+        uint64_t* key = reinterpret_cast<uint64_t*>(rec);
+        sort_list<kLongThreads, true>(cut + start, m,
+                                      SortArrays<true>{key, reinterpret_cast<uint32_t*>(key + n),
+                                                       reinterpret_cast<uint32_t*>(scratch + 16 * static_cast<size_t>(n))},
+                                      M.list.S, tile, keys + start, vals + start);
+        start += m;
+        ++s0;
+      }
+      __syncthreads();  // the next piece reuses the arrays
+    }
+  }
+  pdl_trigger();
+}
+static_assert(kLongShared < 65536, "16-bit bucket counts in shared memory");
+static_assert(4ull * bucket_words<true>(kLongShared + 1) <= 16ull * (kLongShared + 1), "a global sort's buckets fit");
+static_assert(kPairGradStride * sizeof(float) >= 48, "pair_grads holds the unsorted records and the scratch");
+
+}  // namespace
+
+cudaError_t launch_tile_bin(const Layout& L, void* ws, cudaStream_t s) {
+  auto* w = static_cast<uint8_t*>(ws);
+  // dynamic shared memory limits, raised once per device (idempotent: threads may race here)
+  static bool ready[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (!ready[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(sizeof(ListSmem<kTileSortShort>)));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_tile_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(sizeof(LongSmem)));
+    if (e != cudaSuccess) return e;
+    ready[dev] = true;
+  }
+  launch_tile_scan(L, ws, s);
+  const int64_t sms = device_sms();
+  // groups of whole views: a group's emission covers every projection block holding its items
+  const int64_t per_view = static_cast<int64_t>(L.Tx) * L.Ty;
+  int64_t b0 = 0;
+  for (int i = 0; i < L.sort_groups; ++i) {
+    const int64_t k0 = static_cast<int64_t>(L.K) * i / L.sort_groups, k1 = static_cast<int64_t>(L.K) * (i + 1) / L.sort_groups;
+    const int64_t b1 = i + 1 == L.sort_groups ? L.n_proj_groups : (k1 * L.N + L.proj_items - 1) / L.proj_items;
+    if (b1 > b0) launch(k_tile_emit, static_cast<unsigned>(b1 - b0), kEmitThreads, 0, s, L, w, b0);
+    b0 = b1;
+    launch(k_tile_sort, static_cast<unsigned>((k1 - k0) * per_view), kShortThreads, sizeof(ListSmem<kTileSortShort>), s,
+           L, w, k0 * per_view);
+  }
+  launch(k_tile_sort_long, static_cast<unsigned>(L.n_tiles < kLongBlocks * sms ? L.n_tiles : kLongBlocks * sms), kLongThreads,
+         sizeof(LongSmem), s, L, w);
+  return cudaGetLastError();
+}
+
+}  // namespace gs
