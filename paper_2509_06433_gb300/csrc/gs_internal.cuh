@@ -35,8 +35,6 @@ constexpr int64_t kTileSortMaxItems = 1 << 25;  // most Gaussians (so list entri
 constexpr int kTileSortShort = 2048;    // longest list sorted by a short-list block
 constexpr int kTileSortGroupItems = 6400000;  // (view, Gaussian) items per emission / sort launch
 constexpr uint32_t kSpinLimit = 1u << 21;  // bounded decoupled look-back (about a second of polling)
-constexpr int kDefaultFwdPx = 2;      // pixels per thread of the compositing kernels when
-constexpr int kDefaultBwdPx = 2;      // gs_config_t leaves the choice to the library
 
 // Workspace status block (first 256 bytes of the workspace).
 struct Status {

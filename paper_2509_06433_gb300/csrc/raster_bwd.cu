@@ -6,7 +6,7 @@ namespace gs {
 namespace {
 
 template <int PX, int CH>
-__global__ void __launch_bounds__(kTilePixels / PX, PX == 4 ? kMinBlocksPx4 : 1) k_raster_bwd(Layout L, uint8_t* __restrict__ ws,
+__global__ void __launch_bounds__(kTilePixels / PX, PX == 4 ? kMinBlocksPx4 : (PX == 2 ? kMinBlocksBwdPx2 : 1)) k_raster_bwd(Layout L, uint8_t* __restrict__ ws,
                                                                  const float* __restrict__ rgb,
                                                                  const float* __restrict__ depth,
                                                                  const float* __restrict__ T_final,
@@ -63,7 +63,7 @@ cudaError_t launch_raster_bwd(const Layout& L, void* ws, const float* rgb, const
     case 128: GS_BWD(P, 128); break; \
     default: GS_BWD(P, 64); break;   \
   }
-  switch (pick_px(L.bwd_px, kDefaultBwdPx)) {
+  switch (pick_px(L.bwd_px, default_px(L, true))) {
     case 1: GS_BWD_CH(1); break;
     case 2: GS_BWD_CH(2); break;
     default: GS_BWD_CH(4); break;

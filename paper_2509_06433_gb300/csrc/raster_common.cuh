@@ -33,13 +33,15 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kAlphaMax = 0.99f;
 constexpr float kAlphaMin = 1.0f / 255.0f;
 constexpr float kTStop = 1e-4f;
-// Resident blocks per SM the compiler must fit at 4 pixels per thread (64 threads): a register
-// budget of 80 per thread (no spills) for the forward and backward kernels, 72 (a few spilled
-// bytes) for the fused forward + backward. The packed pixel pairs leave the compositing loops
-// bound by instruction latency as much as by issue, and more resident blocks hide more of it
-// (the fused kernel at aerial2m: 6.68 ms at 10 blocks, 6.15 at 12, 6.00 at 14).
+// Resident blocks per SM the compiler must fit: at 4 pixels per thread (64 threads) a register budget
+// of 80 per thread for the forward and backward kernels, 64 (a few spilled bytes) for the fused
+// forward + backward; at 2 (128 threads) 64 for the kernels with a backward sweep. The loops are bound by
+// instruction issue and latency together, and more resident blocks hide more of the latency (fused
+// kernel, 16 aerial views of 1280x720: 3.89 ms at 14 blocks, 3.84 at 16; at 2 pixels per thread 5.24 ms
+// without the budget, 5.03 with 8 blocks; the forward alone is 3% slower with it).
 constexpr int kMinBlocksPx4 = 12;
-constexpr int kMinBlocksFusedPx4 = 14;
+constexpr int kMinBlocksFusedPx4 = 16;
+constexpr int kMinBlocksBwdPx2 = 8;
 constexpr int kFwdChunk = 128;  // splats staged per forward chunk (default; 64 and 256 also built)
 constexpr int kBwdChunk = 64;   // splats staged per backward chunk (default; 32 and 128 also built)
 
@@ -86,11 +88,14 @@ __device__ __forceinline__ typename Vec<W>::T bcast(float x) {
   if constexpr (W == 1) return x;
   else return make_float2(x, x);
 }
-// Staged splat: A = (x, y, qa, qb), B = (qc, opacity, depth, log2 opacity), C = (r, g, b, -) where
+// Staged splat: A = (x, y, qa, qb), B = (qc, opacity, depth, log2 opacity), C = -(r, g, b, depth) where
 // (x, y) is the 2D mean relative to the tile origin and power * log2(e) = qa dx^2 + qb dx dy + qc dy^2.
 // rows: bit r is set when the splat's ellipse {opacity * 2^power >= 1/255}, widened by a safety
 // margin, meets the pixel-centre row y = r + 0.5 of the tile within the columns [0.5, 15.5]. A
-// warp none of whose rows is set skips the splat without changing any decision.
+// warp none of whose rows is set skips the splat without changing any decision. Bit 16 (kChecked)
+// is set unless the splat is proven (plain_splat) to need neither the clamp at 0.99 nor the power
+// <= 0 test at any pixel of the tile; the loops leave both out for the others (most splats).
+constexpr uint32_t kChecked = 1u << 16;
 template <int CH>
 struct Stage {
   float4 A[CH], B[CH], C[CH];
@@ -110,6 +115,20 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// Whether alpha = raw and power <= 0 at every pixel centre of the tile, for a splat with Qa, Qc > 0
+// and Qa Qc - (Qb / 2)^2 = D > 0. The clamp: raw <= opacity (1 + a few ulp) <= 0.981. The power: with
+// S = Qa dx^2 + Qc dy^2 and rho = |Qb| / (2 sqrt(Qa Qc)), the exact exponent is at most lo - (1 - rho) S,
+// and evaluating it (splat_exponent) errs by at most 2^-24 (4 S + |lo|) before the last rounding, which
+// cannot carry it past the representable lo; |lo| <= 8 where any pixel reaches 1/255. So e <= lo holds when
+// kappa = D / (2 Qa Qc) <= 1 - rho is >= 2e-4 and kappa S >= 2e-6, S taken at the column and the row of
+// pixel centres nearest to the mean (the margins also cover the approximate quotient).
+__device__ __forceinline__ bool plain_splat(float mx, float my, float Qa, float Qc, float D, float opacity) {
+  const float kappa = __fdividef(0.5f * D, Qa * Qc);
+  const float ex = mx - 0.5f - fminf(fmaxf(rintf(mx - 0.5f), 0.0f), 15.0f);
+  const float ey = my - 0.5f - fminf(fmaxf(rintf(my - 0.5f), 0.0f), 15.0f);
+  const float S = Qa * ex * ex + Qc * ey * ey;
+  return opacity <= 0.98f && kappa >= 2e-4f && kappa * S >= 2e-6f && S < 1e30f;
+}
 __device__ __forceinline__ uint32_t splat_rows(float mx, float my, float Qa, float Qb, float Qc, float opacity) {
   const float tau0 = __log2f(255.0f * opacity);
   const float tau = tau0 + 0.02f * fabsf(tau0) + 2e-4f;
@@ -118,9 +137,9 @@ __device__ __forceinline__ uint32_t splat_rows(float mx, float my, float Qa, flo
   const float h = 0.5f * Qb;
   const float p1 = Qa * Qc, p2 = h * h;
   const float D = (p1 - p2) + (fmaf(Qa, Qc, -p1) - fmaf(h, h, -p2));
-  if (!(Qa > 0.0f) || !(Qc > 0.0f) || !(D > 0.0f)) return 0xffffu;
+  if (!(Qa > 0.0f) || !(Qc > 0.0f) || !(D > 0.0f)) return 0xffffu | kChecked;
   const float hx = sqrt_approx(__fdividef(tau * Qc, D)), hy = sqrt_approx(__fdividef(tau * Qa, D));
-  if (!(hx < 1e7f) || !(hy < 1e7f)) return 0xffffu;
+  if (!(hx < 1e7f) || !(hy < 1e7f)) return 0xffffu | kChecked;
   constexpr float xa = 0.5f - 0.05f, xb = 15.5f + 0.05f;
   if (mx + hx < xa || mx - hx > xb) return 0u;
   const float sl = __fdividef(h, Qa);  // the ellipse's widest chord at height dy is centred on mx - sl dy
@@ -137,7 +156,8 @@ __device__ __forceinline__ uint32_t splat_rows(float mx, float my, float Qa, flo
   const float r0 = fmaxf(ceilf(my + dn - mm - 0.5f), 0.0f);
   const float r1 = fminf(floorf(my + up + mm - 0.5f), 15.0f);
   if (r0 > r1) return 0u;  // (a NaN bound leaves its side at the tile edge)
-  return (2u << static_cast<int>(r1)) - (1u << static_cast<int>(r0));
+  const uint32_t checked = plain_splat(mx, my, Qa, Qc, D, opacity) ? 0u : kChecked;
+  return ((2u << static_cast<int>(r1)) - (1u << static_cast<int>(r0))) | checked;
 }
 
 template <int CH>
@@ -154,7 +174,7 @@ __device__ __forceinline__ uint32_t stage_splat(Stage<CH>& S, int j, const Layou
   const float lo = __log2f(co.w);
   S.A[j] = make_float4(x, y, qa, qb);
   S.B[j] = make_float4(qc, co.w, cn.w, lo);
-  S.C[j] = make_float4(co.x, co.y, co.z, 0.0f);
+  S.C[j] = make_float4(-co.x, -co.y, -co.z, -cn.w);
   S.rows[j] = splat_rows(x, y, -qa, -qb, -qc, co.w);
   return gid;
 }
@@ -165,7 +185,8 @@ __device__ __forceinline__ uint32_t stage_splat(Stage<CH>& S, int j, const Layou
 //   c1 = qb dx,   c0 = qa dx^2 + log2(opacity),
 // and per pixel row at offset dy the exponent  e = (qc dy + c1) dy + c0 = power log2(e) + log2(o),
 // so raw = 2^e = opacity * exp(power) costs two FMAs and one ex2. The splat is kept at the pixel
-// (not skipped) when power <= 0, i.e. e <= log2(o), and alpha = min(raw, 0.99) >= 1/255.
+// (not skipped) when power <= 0, i.e. e <= log2(o), and alpha = min(raw, 0.99) >= 1/255; for a splat
+// without kChecked both hold as raw >= 1/255 and alpha = raw.
 // The offsets are formed as additions of the negated pixel centre (exact small integers + 0.5),
 // which round exactly as the subtractions would.
 template <int W>
@@ -204,6 +225,12 @@ __device__ __forceinline__ TileCoord tile_coord(const Layout& L, int64_t tile_g)
   return c;
 }
 
+// Pixels per thread when the caller leaves the choice to the library: 4 unless the grid is small, where
+// 2 spreads a tile over twice the warps. With a backward sweep from 1024 tiles on (loss-fused forward +
+// backward, us at 2 / 4 pixels: 672 tiles 133 / 150, 1200 tiles 160 / 150 and 145 / 123, 4032 tiles 195 /
+// 168); forward only from 4000 (300 tiles 28.6 / 36.8, 1200 55 / 53, 3600 with uneven lists 112 / 127,
+// 4032 60 / 58, 9600 236 / 201).
+int default_px(const Layout& L, bool backward) { return L.n_tiles >= (backward ? 1024 : 4000) ? 4 : 2; }
 int pick_px(int requested, int fallback) { return (requested == 1 || requested == 2 || requested == 4) ? requested : fallback; }
 // chunk depth: a power of two in [lo, hi], else the default
 int pick_chunk(int requested, int lo, int hi, int fallback) {

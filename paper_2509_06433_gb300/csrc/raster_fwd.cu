@@ -9,13 +9,11 @@ namespace gs {
 namespace {
 
 // ============================================================================ forward
-// Per pixel, amin is the opacity a splat must reach to be kept: 1/255 while the pixel is
-// open, +inf once it has stopped (or lies outside the image), so a stopped pixel skips every
-// later splat without a separate flag. A kept splat that does not stop the pixel is blended
-// through ae = alpha (else ae = 0): w = ae T and T <- T - ae T leave every accumulator bit for
-// bit unchanged when ae = 0, so the blend needs no selects. STATS = true also counts the
-// evaluations (list entries examined, including the one that stops a pixel) and the blended
-// ones; the decisions and outputs are the same.
+// A pixel that has stopped (or lies outside the image) moves to y = -inf: every later splat's exponent
+// is then -inf (or not a number), so the pixel skips it without a separate flag. A kept splat that does not stop the pixel is blended
+// through alpha, any other through 0, which leaves T and every accumulator bit for bit unchanged,
+// so the blend needs no selects. STATS = true also counts the evaluations (list entries examined,
+// including the one that stops a pixel) and the blended ones; the decisions and outputs are the same.
 // L1 loss fused into the forward pass (LOSS = true): the targets, the gradient images it
 // writes, per-tile partial sums and the block counter that elects the last block to finish,
 // which sums the partials in tile order into *d_loss.
@@ -72,7 +70,8 @@ struct FwdSmemOf<PX, CH, 0> {
 // grids that fit on the GPU in one wave anyway, where each block's own latency sets the time.
 template <int PX, int CH, bool STATS, bool LOSS, bool OCC = false, int CHB = 0, bool MANY = true>
 __global__ void __launch_bounds__(kTilePixels / PX,
-                                  (PX == 4 && MANY) ? (CHB > 0 ? kMinBlocksFusedPx4 : kMinBlocksPx4) : 1)
+                                  PX == 4 && MANY ? (CHB > 0 ? kMinBlocksFusedPx4 : kMinBlocksPx4)
+                                                  : (PX == 2 && CHB > 0 ? kMinBlocksBwdPx2 : 1))
     k_raster_fwd(Layout L, RasterWs<CHB> __restrict__ ws, float* __restrict__ out_rgb, float* __restrict__ out_depth,
                  float* __restrict__ out_T, int32_t* __restrict__ out_last, uint64_t* __restrict__ evals_out,
                  uint64_t* __restrict__ blended_out, FusedLoss F, Occlusion O) {
@@ -96,12 +95,11 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   constexpr int W = PX >= 2 ? 2 : 1, G = PX / W;  // pixel q is component q % W of group q / W
   using V = typename Vec<W>::T;
   V T[G], cr[G], cg[G], cb[G], cd[G], npy[G];
-  float amin[PX];
   int32_t last[PX], stop_at[PX];
   float zmax[PX];
   uint32_t blended = 0;
   bool all_done = true;
-  const V npx = bcast<W>(-pxc), one = bcast<W>(1.0f), zero = bcast<W>(0.0f), minus1 = bcast<W>(-1.0f);
+  const V npx = bcast<W>(-pxc), one = bcast<W>(1.0f), zero = bcast<W>(0.0f);
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     T[g] = one;
@@ -114,7 +112,7 @@ __global__ void __launch_bounds__(kTilePixels / PX,
     last[q] = 0;
     stop_at[q] = -1;
     const bool outside = !(px < L.W && py + q < L.H);
-    amin[q] = outside ? kInf : kAlphaMin;
+    if (outside) set_comp(npy[q / W], q % W, kInf);
     zmax[q] = kInf;
     if (OCC && !outside) zmax[q] = O.depth[tc.k * static_cast<int64_t>(L.H) * L.W + static_cast<int64_t>(py + q) * L.W + px];
     all_done = all_done && outside;
@@ -136,6 +134,74 @@ __global__ void __launch_bounds__(kTilePixels / PX,
       }
     }
   }
+  // One splat of the staged chunk (list position pos): FULL evaluates the clamp and the power test
+  // too (and the occlusion). The blend works on
+  // -alpha (na) and the staged negated colours: T (1 - alpha) = fma(T, na, T) and c alpha T =
+  // (-c)(na T) are the same roundings as with positive operands, without a negated copy of T.
+  const int lane = threadIdx.x & 31;
+  auto splat = [&](auto full, int j, int pos) {
+    constexpr bool FULL = decltype(full)::value;
+    const float4 A = S.A[j], B = S.B[j], C = S.C[j];
+    const Column<W> col = splat_column<W>(A, B, npx);
+    const V Ay = bcast<W>(A.y);
+    V na[G], Tn[G];
+    bool keep[PX];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const V e = splat_exponent<W>(B, col, vadd(Ay, npy[g]));
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const int q = g * W + i;
+        const float raw = ex2_approx(comp(e, i));
+        const float a = FULL ? fminf(raw, kAlphaMax) : raw;
+        keep[q] = a >= kAlphaMin;
+        if (FULL) keep[q] = keep[q] && comp(e, i) <= B.w;
+        if (OCC) keep[q] = keep[q] && !(B.z >= zmax[q]);  // a splat at or behind the surface
+        set_comp(na[g], i, keep[q] ? -a : 0.0f);
+      }
+      Tn[g] = vfma(T[g], na[g], T[g]);
+    }
+    // a pixel stops before the splat that would leave T < 1e-4 (once per pixel, so the changes are
+    // made in a warp-uniform branch; a skipped splat leaves T, which is never below 1e-4)
+    bool event = false;
+    {
+      float low = comp(Tn[0], 0);
+#pragma unroll
+      for (int q = 1; q < PX; ++q) low = fminf(low, comp(Tn[q / W], q % W));
+      event = low < kTStop;
+    }
+    if (OCC) {
+#pragma unroll
+      for (int q = 0; q < PX; ++q) event = event || (B.z >= zmax[q] && comp(npy[q / W], q % W) != kInf);
+    }
+    if (__any_sync(0xffffffffu, event)) {
+#pragma unroll
+      for (int q = 0; q < PX; ++q) {
+        const bool stop = comp(Tn[q / W], q % W) < kTStop;
+        keep[q] = keep[q] && !stop;
+        set_comp(na[q / W], q % W, stop ? 0.0f : comp(na[q / W], q % W));
+        set_comp(npy[q / W], q % W, stop || (OCC && B.z >= zmax[q]) ? kInf : comp(npy[q / W], q % W));
+        if (STATS) stop_at[q] = stop ? pos : stop_at[q];
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) Tn[g] = vfma(T[g], na[g], T[g]);
+    }
+    const V nR = bcast<W>(C.x), nG = bcast<W>(C.y), nB = bcast<W>(C.z), nZ = bcast<W>(C.w);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const V nw = vmul(na[g], T[g]);
+      cr[g] = vfma(nR, nw, cr[g]);
+      cg[g] = vfma(nG, nw, cg[g]);
+      cb[g] = vfma(nB, nw, cb[g]);
+      cd[g] = vfma(nZ, nw, cd[g]);
+      T[g] = Tn[g];
+    }
+#pragma unroll
+    for (int q = 0; q < PX; ++q) {
+      last[q] = keep[q] ? pos + 1 : last[q];
+      if (STATS) blended += keep[q] ? 1u : 0u;
+    }
+  };
   for (uint32_t base = rg.x; base < rg.y; base += CH) {
     if (__syncthreads_count(!all_done) == 0) break;
     for (int jj = threadIdx.x; jj < CH; jj += kThreads) {
@@ -145,57 +211,31 @@ __global__ void __launch_bounds__(kTilePixels / PX,
     __syncthreads();
     const int n = min(CH, static_cast<int>(rg.y - base));
     const int pos0 = static_cast<int>(base - rg.x);
-    for (int j = 0; j < n; ++j) {
-      if ((j & 7) == 0) {  // warp-uniform early exit, checked every 8 splats (extra ones are no-ops)
+    // the splats that meet the warp's rows, 32 at a time (the loop runs over the set bits only; it
+    // ends early when every pixel of the warp has stopped, looked at after every 8 list positions)
+    bool done = __all_sync(0xffffffffu, all_done);
+#pragma unroll 1
+    for (int w0 = 0; w0 < n && !done; w0 += 32) {
+      const uint32_t r = w0 + lane < n ? S.rows[w0 + lane] : 0u;
+      uint32_t visit = __ballot_sync(0xffffffffu, (r & wrows) != 0);
+      const uint32_t checked = __ballot_sync(0xffffffffu, (r & kChecked) != 0);
+#pragma unroll 1
+      for (int k = 0; visit && !done; k += 8) {
+        uint32_t v = visit & (0xffu << k);
+        visit &= ~(0xffu << k);
+        int j = __ffs(v) - 1;
+#pragma unroll 1
+        while (j >= 0) {
+          v &= v - 1;
+          const int next = __ffs(v) - 1;  // (found ahead of the splat's own chain)
+          if (OCC || ((checked >> j) & 1u)) splat(std::true_type{}, w0 + j, pos0 + w0 + j);
+          else splat(std::false_type{}, w0 + j, pos0 + w0 + j);
+          j = next;
+        }
         all_done = true;
 #pragma unroll
-        for (int q = 0; q < PX; ++q) all_done = all_done && (amin[q] == kInf);
-        if (__all_sync(0xffffffffu, all_done)) break;
-      }
-      if (!(S.rows[j] & wrows)) continue;
-      const float4 A = S.A[j], B = S.B[j], C = S.C[j];
-      const Column<W> col = splat_column<W>(A, B, npx);
-      const V cR = bcast<W>(C.x), cG = bcast<W>(C.y), cB = bcast<W>(C.z), cZ = bcast<W>(B.z), Ay = bcast<W>(A.y);
-      const int pos = pos0 + j;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const V e = splat_exponent<W>(B, col, vadd(Ay, npy[g]));
-        const V nT = vmul(T[g], minus1);
-        V alpha;
-        bool keep[W];
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-          const int q = g * W + i;
-          const float a = fminf(ex2_approx(comp(e, i)), kAlphaMax);
-          set_comp(alpha, i, a);
-          keep[i] = (comp(e, i) <= B.w) && (a >= amin[q]);
-        }
-        const V Tn = vfma(nT, alpha, T[g]);  // T (1 - alpha)
-        V ae;  // alpha for a blended splat, else 0 (then w = 0 and T, the sums stay bit for bit)
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-          const int q = g * W + i;
-          bool kp = keep[i], behind = false;
-          if (OCC) {
-            behind = B.z >= zmax[q];  // the splat's camera depth at or behind the surface
-            kp = kp && !behind;
-          }
-          const bool stop = kp && (comp(Tn, i) < kTStop);
-          const bool blend = kp && !stop;
-          set_comp(ae, i, blend ? comp(alpha, i) : 0.0f);
-          last[q] = blend ? pos + 1 : last[q];
-          amin[q] = (stop || behind) ? kInf : amin[q];
-          if (STATS) {
-            stop_at[q] = stop ? pos : stop_at[q];
-            blended += blend ? 1u : 0u;
-          }
-        }
-        const V w = vmul(ae, T[g]);
-        cr[g] = vfma(cR, w, cr[g]);
-        cg[g] = vfma(cG, w, cg[g]);
-        cb[g] = vfma(cB, w, cb[g]);
-        cd[g] = vfma(cZ, w, cd[g]);
-        T[g] = vfma(nT, ae, T[g]);
+        for (int q = 0; q < PX; ++q) all_done = all_done && comp(npy[q / W], q % W) == kInf;
+        done = __all_sync(0xffffffffu, all_done);
       }
     }
   }
@@ -347,7 +387,7 @@ cudaError_t launch_raster_fwd_l1_bwd(const Layout& L, void* ws, float* rgb, floa
   uint64_t *ev = &st->evals, *cp = &st->composited;
   const FusedLoss F{loss.rgb_t, loss.depth_t, loss.g_rgb, loss.g_depth, at<float>(ws, L.tile_loss), &st->loss_ctr,
                     loss.d_loss};
-  const int px = pick_px(L.fwd_px, kDefaultFwdPx);
+  const int px = pick_px(L.fwd_px, default_px(L, true));
   const int ch = pick_chunk(L.fwd_chunk, 64, 256, kFwdChunk);
   // the backward phase stages kBwdChunk splats per chunk (the chunk depth changes no result); at 4
   // pixels per thread, a grid that the variant without the blocks-per-SM register budget runs in
@@ -408,7 +448,7 @@ cudaError_t launch_raster_fwd(const Layout& L, void* ws, float* rgb, float* dept
   if (loss)
     F = FusedLoss{loss->rgb_t, loss->depth_t, loss->g_rgb, loss->g_depth, at<float>(ws, L.tile_loss), &st->loss_ctr,
                   loss->d_loss};
-  const int px = pick_px(L.fwd_px, kDefaultFwdPx);
+  const int px = pick_px(L.fwd_px, default_px(L, loss != nullptr));
   const int ch = pick_chunk(L.fwd_chunk, 64, 256, kFwdChunk);
 #define GS_FWD(P, C, ST, LO)                                                                                  \
   launch(k_raster_fwd<P, C, ST, LO>, grid, kTilePixels / P, cap_smem(k_raster_fwd<P, C, ST, LO>, L.raster_bps), s, \

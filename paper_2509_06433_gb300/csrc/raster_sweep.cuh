@@ -3,6 +3,8 @@
 // opacity test it shares with the forward.
 #pragma once
 
+#include <type_traits>
+
 #include "raster_common.cuh"
 
 namespace gs {
@@ -58,6 +60,7 @@ struct BwdSmem {
   Stage<CH> S;
   uint32_t slot[CH];
   float part[kWarps][CH][10];
+  uint32_t written[kWarps][CH / 32];  // splats of the chunk whose part a warp has written
   int maxlast[kWarps];
 };
 
@@ -104,8 +107,8 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
   uint32_t* pair_valid = at<uint32_t>(ws, L.pair_valid);
   constexpr int W = PX >= 2 ? 2 : 1, G = PX / W;  // pixel q is component q % W of group q / W
   using V = typename Vec<W>::T;
-  const V npx = bcast<W>(-pxc), zero = bcast<W>(0.0f), minus1 = bcast<W>(-1.0f);
-  V T[G], npy[G], Sgv[G], hTv[G], grv[G], ggv[G], gbv[G], gdv[G];
+  const V npx = bcast<W>(-pxc), zero = bcast<W>(0.0f);
+  V T[G], npy[G], nS[G], grv[G], ggv[G], gbv[G], gdv[G];
   int wl = 0;
 #pragma unroll
   for (int g = 0; g < G; ++g) {
@@ -114,8 +117,7 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
     for (int i = 0; i < W; ++i) {
       const int q = g * W + i;
       set_comp(npy[g], i, -(pyc + static_cast<float>(q)));
-      set_comp(Sgv[g], i, Sg[q]);
-      set_comp(hTv[g], i, hT[q]);
+      set_comp(nS[g], i, HT ? -(Sg[q] + hT[q]) : -Sg[q]);
       set_comp(grv[g], i, gr[q]);
       set_comp(ggv[g], i, gg[q]);
       set_comp(gbv[g], i, gb[q]);
@@ -136,6 +138,80 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
   const bool writer = reduce10_writer(lane);
   constexpr float kLn2 = 0.6931471805599453f;
 
+  // One splat of the staged chunk at list position pos; returns whether a pixel of the warp keeps it.
+  // FULL evaluates the clamp at 0.99 and the power test too (see kChecked).
+  auto splat = [&](auto full, int j, int pos) -> bool {
+    constexpr bool FULL = decltype(full)::value;
+    const float4 A = M.S.A[j], B = M.S.B[j];
+    const Column<W> col = splat_column<W>(A, B, npx);
+    const V Ay = bcast<W>(A.y);
+    // phase 1: opacity and keep/skip decision for the thread's pixels
+    V dy[G];
+    float raw[PX];
+    bool okq[PX];
+    bool contrib = false;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      dy[g] = vadd(Ay, npy[g]);
+      const V e = splat_exponent<W>(B, col, dy[g]);
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const int q = g * W + i;
+        raw[q] = ex2_approx(comp(e, i));
+        okq[q] = raw[q] >= kAlphaMin && pos < last[q];
+        if (FULL) okq[q] = okq[q] && comp(e, i) <= B.w;
+        contrib = contrib || okq[q];
+      }
+    }
+    // phase 2 (skipped when no pixel of the warp keeps the splat): gradient terms, two pixels
+    // per packed instruction. With na = -alpha of a kept splat (else 0), nw = na T is minus its weight,
+    // nc = -(colour . upstream gradient) and nS minus the weighted colour behind the splat, which
+    // becomes nS + nw nc; then dL/dpower = w (c - S / T') with T' = T (1 - alpha), i.e. nw (nc - nS / T').
+    // The colour-gradient sums are kept negated.
+    if (!__any_sync(0xffffffffu, contrib)) return false;
+    const float4 C = M.S.C[j];
+    const V nR = bcast<W>(C.x), nG = bcast<W>(C.y), nB = bcast<W>(C.z), nZ = bcast<W>(C.w);
+    V P0 = zero, P1 = zero, P2 = zero, ncz = zero, ncr = zero, ncg = zero, ncb = zero;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      V na, nr;
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const int q = g * W + i;
+        const float a = FULL ? fminf(raw[q], kAlphaMax) : raw[q];
+        set_comp(na, i, okq[q] ? -a : 0.0f);
+      }
+      const V nw = vmul(na, T[g]);
+      const V Tn = vfma(T[g], na, T[g]);
+      const V nc = vfma(nZ, gdv[g], vfma(nB, gbv[g], vfma(nG, ggv[g], vmul(nR, grv[g]))));
+      nS[g] = vfma(nw, nc, nS[g]);
+#pragma unroll
+      for (int i = 0; i < W; ++i) set_comp(nr, i, rcp_approx(-comp(Tn, i)));
+      V dpow = vmul(nw, vfma(nS[g], nr, nc));
+      if (FULL) {  // the clamp passes no gradient
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+          if (raw[g * W + i] > kAlphaMax) set_comp(dpow, i, 0.0f);
+      }
+      const V ydp = vmul(dy[g], dpow);
+      P0 = vadd(P0, dpow);
+      P1 = vadd(P1, ydp);
+      P2 = vfma(dy[g], ydp, P2);
+      ncz = vfma(nw, gdv[g], ncz);
+      ncr = vfma(nw, grv[g], ncr);
+      ncg = vfma(nw, ggv[g], ncg);
+      ncb = vfma(nw, gbv[g], ncb);
+      T[g] = Tn;
+    }
+    const float p0 = hsum(P0), p1 = hsum(P1);
+    const float dx = comp(col.dx, 0);
+    const float dxP0 = dx * p0;
+    const float v[10] = {dxP0, p1, dx * dxP0, dx * p1, hsum(P2), hsum(ncz), p0, hsum(ncr), hsum(ncg), hsum(ncb)};
+    const float r = warp_reduce10(v, lane);
+    if (writer) M.part[warp][j][idx] = r;
+    return true;
+  };
+
   for (uint32_t base = rg.x; base < stop; base += CH) {
     for (int jj = threadIdx.x; jj < CH; jj += kThreads) {
       const uint32_t i = base + jj;
@@ -144,89 +220,43 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
         M.slot[jj] = slots[i];
       }
     }
-    for (int e = threadIdx.x; e < kWarps * CH * 10; e += kThreads) (&M.part[0][0][0])[e] = 0.0f;
     __syncthreads();
     const int n = min(CH, static_cast<int>(stop - base));
     const int pos0 = static_cast<int>(base - rg.x);
     const int nw = min(n, warp_last - pos0);  // splats of this chunk this warp must visit
-    for (int j = 0; j < nw; ++j) {
-      if (!(M.S.rows[j] & wrows)) continue;
-      const float4 A = M.S.A[j], B = M.S.B[j];
-      const Column<W> col = splat_column<W>(A, B, npx);
-      const V Ay = bcast<W>(A.y);
-      const int pos = pos0 + j;
-      // phase 1: opacity and keep/skip decision for the thread's pixels
-      V dy[G], alpha[G];
-      float raw[PX];
-      bool okq[PX];
-      bool contrib = false;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        dy[g] = vadd(Ay, npy[g]);
-        const V e = splat_exponent<W>(B, col, dy[g]);
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-          const int q = g * W + i;
-          raw[q] = ex2_approx(comp(e, i));
-          const float a = fminf(raw[q], kAlphaMax);
-          set_comp(alpha[g], i, a);
-          okq[q] = (comp(e, i) <= B.w) && (a >= kAlphaMin) && (pos < last[q]);
-          contrib = contrib || okq[q];
-        }
+    // the splats that meet the warp's rows, 32 at a time (the loop runs over the set bits only)
+#pragma unroll 1
+    for (int w0 = 0; w0 < CH; w0 += 32) {
+      const uint32_t r = w0 + lane < nw ? M.S.rows[w0 + lane] : 0u;
+      uint32_t visit = __ballot_sync(0xffffffffu, (r & wrows) != 0);
+      const uint32_t checked = __ballot_sync(0xffffffffu, (r & kChecked) != 0);
+      uint32_t written = 0;
+      int b = __ffs(visit) - 1;
+#pragma unroll 1
+      while (b >= 0) {
+        visit &= visit - 1;
+        const int next = __ffs(visit) - 1;
+        const bool some = ((checked >> b) & 1u) ? splat(std::true_type{}, w0 + b, pos0 + w0 + b)
+                                                : splat(std::false_type{}, w0 + b, pos0 + w0 + b);
+        if (some) written |= 1u << b;
+        b = next;
       }
-      // phase 2 (skipped when no pixel of the warp keeps the splat): gradient terms, two pixels
-      // per packed instruction. The colour-gradient sums are kept negated (nw = -w).
-      if (!__any_sync(0xffffffffu, contrib)) continue;
-      const float4 C = M.S.C[j];
-      const V cR = bcast<W>(C.x), cG = bcast<W>(C.y), cB = bcast<W>(C.z), cZ = bcast<W>(B.z);
-      V P0 = zero, P1 = zero, P2 = zero, ncz = zero, ncr = zero, ncg = zero, ncb = zero;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        // aok = alpha for a kept splat, else 0: then w = 0 and Sg, T stay unchanged;
-        // oal = alpha where the gradient passes (kept and not clamped at 0.99), else 0
-        V aok, oal, nr;
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-          const int q = g * W + i;
-          const float a = comp(alpha[g], i);
-          set_comp(aok, i, okq[q] ? a : 0.0f);
-          set_comp(oal, i, (okq[q] && !(raw[q] > kAlphaMax)) ? a : 0.0f);
-          set_comp(nr, i, rcp_approx(a - 1.0f));  // -1 / (1 - alpha)
-        }
-        const V nT = vmul(T[g], minus1);
-        const V nw = vmul(aok, nT);
-        const V cgz = vfma(cZ, gdv[g], vfma(cB, gbv[g], vfma(cG, ggv[g], vmul(cR, grv[g]))));
-        const V sg = vfma(cgz, nw, Sgv[g]);  // colour/depth behind this splat, weighted by dL/dpixel
-        const V dalpha = vfma(T[g], cgz, vmul(HT ? vadd(sg, hTv[g]) : sg, nr));
-        const V dpow = vmul(oal, dalpha);
-        const V ydp = vmul(dy[g], dpow);
-        P0 = vadd(P0, dpow);
-        P1 = vadd(P1, ydp);
-        P2 = vfma(dy[g], ydp, P2);
-        ncz = vfma(nw, gdv[g], ncz);
-        ncr = vfma(nw, grv[g], ncr);
-        ncg = vfma(nw, ggv[g], ncg);
-        ncb = vfma(nw, gbv[g], ncb);
-        Sgv[g] = sg;
-        T[g] = vfma(nT, aok, T[g]);
-      }
-      const float p0 = hsum(P0), p1 = hsum(P1);
-      const float dx = comp(col.dx, 0);
-      const float dxP0 = dx * p0;
-      const float v[10] = {dxP0, p1, dx * dxP0, dx * p1, hsum(P2), hsum(ncz), p0, hsum(ncr), hsum(ncg), hsum(ncb)};
-      const float r = warp_reduce10(v, lane);
-      if (writer) M.part[warp][j][idx] = r;
+      if (lane == 0) M.written[warp][w0 / 32] = written;
     }
     __syncthreads();
     for (int jj = threadIdx.x; jj < n; jj += kThreads) {
       float R[10];
+      bool any = false;
 #pragma unroll
-      for (int q = 0; q < 10; ++q) {
-        float acc = 0.0f;
+      for (int q = 0; q < 10; ++q) R[q] = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) acc += M.part[w][jj][q];
-        R[q] = acc;
+      for (int w = 0; w < kWarps; ++w) {
+        if (!((M.written[w][jj >> 5] >> (jj & 31)) & 1u)) continue;
+        any = true;
+#pragma unroll
+        for (int q = 0; q < 10; ++q) R[q] += M.part[w][jj][q];
       }
+      if (!any) continue;  // no pixel keeps the splat: no record (its gradient is zero)
       // R = (sum dx P0, sum P1, sum dx^2 P0, sum dx P1, sum P2, -dz, sum P0, -dr, -dg, -db)
       const float qa = M.S.A[jj].z, qb = M.S.A[jj].w, qc = M.S.B[jj].x, op = M.S.B[jj].y;
       const float du = kLn2 * (2.0f * qa * R[0] + qb * R[1]);
@@ -242,7 +272,7 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
     }
     __syncthreads();
   }
-  // pairs behind every pixel's last contributor get no record: their bit stays clear
+  // pairs that no pixel keeps or behind every pixel's last contributor get no record: their bit stays clear
 }
 
 }  // namespace
