@@ -6,9 +6,9 @@
 // planes and C1 = (0.01 R)^2, C2 = (0.03 R)^2; an image's SSIM is the mean of its map.
 //
 // Both are deterministic: every block writes one partial sum to the caller's scratch, and one
-// block per image adds its partials in a fixed order (in FP64). SSIM stages a 26 x 26 halo tile
-// of both planes in shared memory, filters the five moments (x, y, x^2, y^2, xy) along x for
-// the 26 rows, then along y for the 16 x 16 outputs.
+// block per image adds its partials in a fixed order (in FP64). SSIM walks down a strip of columns,
+// one column per thread: the five moments (x, y, x^2, y^2, xy) filtered along x are formed per row
+// from a staged row group, and the last 11 rows of them, in registers, give the window sums.
 #include <math.h>
 
 #include "gs_internal.cuh"
@@ -18,10 +18,8 @@ namespace {
 
 constexpr int kMetThreads = 256;
 constexpr int kPsnrChunk = 8192;  // values per PSNR block
-constexpr int kSsimTile = 16;
 constexpr int kSsimTaps = 11;
 constexpr int kSsimRad = kSsimTaps / 2;
-constexpr int kSsimIn = kSsimTile + 2 * kSsimRad;  // 26
 
 struct Window {
   float w[kSsimTaps];
@@ -82,68 +80,113 @@ __global__ void __launch_bounds__(kMetThreads) k_psnr_final(const float* __restr
   }
 }
 
-// one block per (16 x 16 tile, plane); plane = image * C + channel
-__global__ void __launch_bounds__(kMetThreads) k_ssim(const float* __restrict__ x, const float* __restrict__ y, int H,
-                                                     int W, int tiles_x, int tiles_per_plane, Window win, float c1,
-                                                     float c2, float* __restrict__ map, float* __restrict__ partials) {
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool in) {  // zero when !in
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One block per (strip of kSsimCols columns x kSsimRows rows, plane); plane = image * C + channel. Thread c
+// owns output column c of the strip and keeps the five x-filtered moments of the last 11 input rows
+// in registers; a group of 11 input rows is staged as (x, y) pairs at a time, so the loop over a group is
+// unrolled and every register index is a constant. Bound by FP32 issue: 11 taps of 5 moments along x
+// and along y per output, two moments per packed instruction. The 16 x 16 tile with shared x-filtered
+// moments it replaces read 90 shared-memory words per output (27 here) and was bound by them: four
+// 672x376 RGB images (both launches) 62 -> 33 us, eight 1280x720 ones 399 -> 167. 34 rows per strip
+// (more blocks, more warm-up): 38 and 179; 128 columns: 38 and 160.
+constexpr int kSsimCols = 64;
+constexpr int kSsimRows = 45;  // output rows per strip: five groups of 11 input rows, less 10 of warm-up
+constexpr int kSsimGroups = (kSsimRows + 2 * kSsimRad) / kSsimTaps;
+static_assert(kSsimGroups * kSsimTaps == kSsimRows + 2 * kSsimRad, "whole groups of input rows");
+
+__global__ void __launch_bounds__(kSsimCols) k_ssim(const float* __restrict__ x, const float* __restrict__ y, int H,
+                                                    int W, int strips_x, int strips_per_plane, Window win, float c1,
+                                                    float c2, float* __restrict__ map, float* __restrict__ partials) {
   pdl_begin();
-  __shared__ float sx[kSsimIn][kSsimIn], sy[kSsimIn][kSsimIn];
-  __shared__ float hm[5][kSsimIn][kSsimTile];
-  __shared__ float s_warp[kMetThreads / 32];
+  constexpr int kIn = kSsimCols + 2 * kSsimRad;
+  __shared__ float2 s_in[2][kSsimTaps][kIn];
+  __shared__ float s_warp[kSsimCols / 32];
   const int64_t plane = blockIdx.y;
-  const int t = blockIdx.x;
-  const int ty0 = (t / tiles_x) * kSsimTile, tx0 = (t % tiles_x) * kSsimTile;
+  const int t = blockIdx.x, col = threadIdx.x;
+  const int y0 = (t / strips_x) * kSsimRows, x0 = (t % strips_x) * kSsimCols;
   const int64_t HW = static_cast<int64_t>(H) * W;
   const float* xp = x + plane * HW;
   const float* yp = y + plane * HW;
-  for (int i = threadIdx.x; i < kSsimIn * kSsimIn; i += kMetThreads) {
-    const int r = i / kSsimIn, c = i - r * kSsimIn;
-    const int gy = ty0 + r - kSsimRad, gx = tx0 + c - kSsimRad;
-    const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-    const int64_t o = static_cast<int64_t>(gy) * W + gx;
-    sx[r][c] = in ? xp[o] : 0.0f;
-    sy[r][c] = in ? yp[o] : 0.0f;
-  }
-  __syncthreads();
-  // along x: the 26 rows x 16 output columns
-  for (int i = threadIdx.x; i < kSsimIn * kSsimTile; i += kMetThreads) {
-    const int r = i / kSsimTile, c = i - r * kSsimTile;
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f, a4 = 0.0f;
+  const int gx = x0 + col;
+  // Group grp's rows go to buffer grp & 1 by asynchronous copies (zeros outside the image), which run
+  // while the group before is filtered: a thread copies its own column, two threads per row the halo.
+  const uint32_t smem0 = static_cast<uint32_t>(__cvta_generic_to_shared(&s_in[0][0][0]));
+  auto copy = [&](int buf, int r, int c, int iy) {
+    const int ix = x0 + c - kSsimRad;
+    const bool in = iy >= 0 && iy < H && ix >= 0 && ix < W;
+    const int64_t o = in ? static_cast<int64_t>(iy) * W + ix : 0;
+    const uint32_t dst = smem0 + static_cast<uint32_t>(((buf * kSsimTaps + r) * kIn + c) * sizeof(float2));
+    cp_async4(dst, xp + o, in);
+    cp_async4(dst + 4, yp + o, in);
+  };
+  auto stage = [&](int grp) {
+    const int iy0 = y0 + grp * kSsimTaps - kSsimRad;
 #pragma unroll
-    for (int a = 0; a < kSsimTaps; ++a) {
-      const float u = sx[r][c + a], v = sy[r][c + a], w = win.w[a];
-      a0 = fmaf(w, u, a0);
-      a1 = fmaf(w, v, a1);
-      a2 = fmaf(w, u * u, a2);
-      a3 = fmaf(w, v * v, a3);
-      a4 = fmaf(w, u * v, a4);
+    for (int r = 0; r < kSsimTaps; ++r) copy(grp & 1, r, col, iy0 + r);
+    for (int i = col; i < 2 * kSsimRad * kSsimTaps; i += kSsimCols) {
+      const int r = i / (2 * kSsimRad);
+      copy(grp & 1, r, kSsimCols + i - r * 2 * kSsimRad, iy0 + r);
     }
-    hm[0][r][c] = a0;
-    hm[1][r][c] = a1;
-    hm[2][r][c] = a2;
-    hm[3][r][c] = a3;
-    hm[4][r][c] = a4;
-  }
-  __syncthreads();
-  // along y: one output pixel per thread
-  const int r = threadIdx.x / kSsimTile, c = threadIdx.x - r * kSsimTile;
-  float mx = 0.0f, my = 0.0f, exx = 0.0f, eyy = 0.0f, exy = 0.0f;
+  };
+  float2 hm[kSsimTaps], hq[kSsimTaps];  // x-filtered (x, y) and (x^2, y^2) of input row r, at r % 11
+  float hc[kSsimTaps];                  // and xy
+  float tot = 0.0f;
+  stage(0);
+  for (int grp = 0; grp < kSsimGroups; ++grp) {
+    cp_async_wait_all();
+    __syncthreads();
+    if (grp + 1 < kSsimGroups && y0 + (grp + 1) * kSsimTaps - kSsimRad < H + kSsimRad) stage(grp + 1);
 #pragma unroll
-  for (int a = 0; a < kSsimTaps; ++a) {
-    const float w = win.w[a];
-    mx = fmaf(w, hm[0][r + a][c], mx);
-    my = fmaf(w, hm[1][r + a][c], my);
-    exx = fmaf(w, hm[2][r + a][c], exx);
-    eyy = fmaf(w, hm[3][r + a][c], eyy);
-    exy = fmaf(w, hm[4][r + a][c], exy);
+    for (int r = 0; r < kSsimTaps; ++r) {
+      float2 m = make_float2(0.0f, 0.0f), q = make_float2(0.0f, 0.0f);
+      float c = 0.0f;
+#pragma unroll
+      for (int a = 0; a < kSsimTaps; ++a) {
+        const float2 u = s_in[grp & 1][r][col + a];
+        const float2 w = make_float2(win.w[a], win.w[a]);
+        m = __ffma2_rn(w, u, m);
+        q = __ffma2_rn(w, __fmul2_rn(u, u), q);
+        c = fmaf(win.w[a], u.x * u.y, c);
+      }
+      hm[r] = m;
+      hq[r] = q;
+      hc[r] = c;
+      // the window of output row gy ends at this input row; its first row is the oldest kept
+      const int gy = y0 + grp * kSsimTaps + r - 2 * kSsimRad;
+      if (grp * kSsimTaps + r < 2 * kSsimRad || gy >= H) continue;
+      float2 mu = make_float2(0.0f, 0.0f), e2 = make_float2(0.0f, 0.0f);
+      float exy = 0.0f;
+#pragma unroll
+      for (int a = 0; a < kSsimTaps; ++a) {
+        const int s = (r + 1 + a) % kSsimTaps;
+        const float2 w = make_float2(win.w[a], win.w[a]);
+        mu = __ffma2_rn(w, hm[s], mu);
+        e2 = __ffma2_rn(w, hq[s], e2);
+        exy = fmaf(win.w[a], hc[s], exy);
+      }
+      const float mx = mu.x, my = mu.y;
+      const float vx = e2.x - mx * mx, vy = e2.y - my * my, cxy = exy - mx * my;
+      const float s = ((2.0f * mx * my + c1) * (2.0f * cxy + c2)) / ((mx * mx + my * my + c1) * (vx + vy + c2));
+      if (gx < W) {
+        if (map) map[plane * HW + static_cast<int64_t>(gy) * W + gx] = s;
+        tot += s;
+      }
+    }
   }
-  const float vx = exx - mx * mx, vy = eyy - my * my, cxy = exy - mx * my;
-  const float s = ((2.0f * mx * my + c1) * (2.0f * cxy + c2)) / ((mx * mx + my * my + c1) * (vx + vy + c2));
-  const int gy = ty0 + r, gx = tx0 + c;
-  const bool valid = gy < H && gx < W;
-  if (valid && map) map[plane * HW + static_cast<int64_t>(gy) * W + gx] = s;
-  const float tot = block_sum(valid ? s : 0.0f, s_warp);
-  if (threadIdx.x == 0) partials[plane * tiles_per_plane + t] = tot;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  if ((col & 31) == 0) s_warp[col >> 5] = tot;
+  __syncthreads();
+  if (col == 0) {
+    float sum = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kSsimCols / 32; ++w) sum += s_warp[w];
+    partials[plane * strips_per_plane + t] = sum;
+  }
 }
 
 __global__ void __launch_bounds__(kMetThreads) k_mean_final(const float* __restrict__ partials, int64_t per_image,
@@ -165,8 +208,13 @@ int64_t psnr_blocks(int32_t C, int32_t H, int32_t W) {
   const int64_t n = static_cast<int64_t>(C) * H * W;
   return (n + kPsnrChunk - 1) / kPsnrChunk;
 }
-int64_t ssim_tiles(int32_t H, int32_t W) {
-  return static_cast<int64_t>((W + kSsimTile - 1) / kSsimTile) * ((H + kSsimTile - 1) / kSsimTile);
+int64_t ssim_strips(int32_t H, int32_t W) {
+  return static_cast<int64_t>((W + kSsimCols - 1) / kSsimCols) * ((H + kSsimRows - 1) / kSsimRows);
+}
+// Partial sums the scratch of gs_metrics_tmp_size holds per plane (one per 16 x 16 tile, of which a strip
+// covers at least one).
+int64_t ssim_scratch(int32_t H, int32_t W) {
+  return static_cast<int64_t>((W + 15) / 16) * ((H + 15) / 16);
 }
 
 }  // namespace
@@ -178,7 +226,7 @@ extern "C" gs_status_t gs_metrics_tmp_size(int32_t images, int32_t channels, int
                                            size_t* bytes) {
   if (!bytes || !dims_ok(images, channels, height, width)) return GS_ERR_INVALID_ARG;
   const int64_t a = images * psnr_blocks(channels, height, width);
-  const int64_t b = static_cast<int64_t>(images) * channels * ssim_tiles(height, width);
+  const int64_t b = static_cast<int64_t>(images) * channels * ssim_scratch(height, width);
   *bytes = static_cast<size_t>(a > b ? a : b) * sizeof(float);
   return GS_OK;
 }
@@ -217,13 +265,13 @@ extern "C" gs_status_t gs_ssim(const float* x, const float* y, int32_t images, i
   for (int a = 0; a < kSsimTaps; ++a) win.w[a] = static_cast<float>(w[a] / sum);
   const float c1 = static_cast<float>((0.01 * data_range) * (0.01 * data_range));
   const float c2 = static_cast<float>((0.03 * data_range) * (0.03 * data_range));
-  const int tiles_x = (width + kSsimTile - 1) / kSsimTile;
-  const int tiles = static_cast<int>(ssim_tiles(height, width));
+  const int strips_x = (width + kSsimCols - 1) / kSsimCols;
+  const int strips = static_cast<int>(ssim_strips(height, width));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   float* part = static_cast<float*>(tmp);
-  launch(k_ssim, dim3(tiles, images * channels), kMetThreads, 0, s, x, y, height, width, tiles_x, tiles, win, c1, c2,
+  launch(k_ssim, dim3(strips, images * channels), kSsimCols, 0, s, x, y, height, width, strips_x, strips, win, c1, c2,
          ssim_map, part);
-  launch(k_mean_final, images, kMetThreads, 0, s, part, static_cast<int64_t>(channels) * tiles,
+  launch(k_mean_final, images, kMetThreads, 0, s, part, static_cast<int64_t>(channels) * strips,
          static_cast<double>(channels) * height * width, ssim);
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
