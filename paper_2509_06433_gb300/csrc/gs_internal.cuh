@@ -473,7 +473,7 @@ __host__ __device__ inline int64_t sort_tiles(int64_t n, int items) {
 // Keys per thread for a sort of up to n keys: small sorts take short tiles, so that enough
 // blocks share the work.
 // keys per thread: small sorts take small tiles (more blocks, shorter per-tile latency)
-inline int pick_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 600000 ? 8 : kSortItems); }
+inline int pick_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 1000000 ? 8 : kSortItems); }
 using SortArgs = SortArgsT<uint64_t>;
 using SortArgs32 = SortArgsT<uint32_t>;
 cudaError_t launch_onesweep(const SortArgs& a, cudaStream_t s);

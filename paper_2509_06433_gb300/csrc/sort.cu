@@ -309,8 +309,9 @@ cudaError_t launch_onesweep(const SortArgs32& a, cudaStream_t s) { return oneswe
 cudaError_t launch_sort_prepare(const SortArgs& a, cudaStream_t s) {
   cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * 256 * a.passes, s);
   cudaMemsetAsync(a.tile_ctr, 0, sizeof(uint32_t) * kMaxSortPasses, s);
-  int64_t blocks = (a.n_host + 255) / 256;
-  if (blocks > 1024) blocks = 1024;
+  // (every block adds its histograms to the global ones: few blocks of many keys)
+  int64_t blocks = (a.n_host + 1023) / 1024;
+  if (blocks > 2 * num_sms()) blocks = 2 * num_sms();
   if (blocks < 1) blocks = 1;
   launch(k_sort_hist, static_cast<unsigned>(blocks), 256, 0, s, a);
   return cudaGetLastError();
