@@ -145,6 +145,7 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
   } else {
     L->stage_ell = take(KN * 32);
     L->stage_meta = take(KN * 16);
+    L->surv_blocks = take(static_cast<size_t>(L->n_proj_groups) * 4);
     L->block_pairs = take(static_cast<size_t>(L->n_proj_groups) * 4);
     L->tile_cursor = take(static_cast<size_t>(L->n_tiles) * kTileSubLists * kCursorStride * 4);
     L->long_tiles = take(static_cast<size_t>(L->n_tiles) * 4);

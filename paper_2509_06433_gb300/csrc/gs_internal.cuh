@@ -17,6 +17,7 @@ constexpr int kProjItemsMax = 2048;   // (view, Gaussian) items per projection b
                                       // this, a power of two, so that there are >= kProjTargetBlocks
 constexpr int kProjTargetBlocks = 1216;
 constexpr int kProjThreads = 256;     // threads of a projection block
+constexpr int kProjViews = 4;         // views whose cameras a projection block keeps in shared memory
 constexpr int kEmitPairs = 1024;      // pairs emitted per emission block
 constexpr int kProjGridCells = 6144;  // largest (Tx+1)(Ty+1) difference grid kept in shared memory
 constexpr int kSortThreads = 256;     // onesweep block
@@ -121,9 +122,10 @@ struct Layout {
   // Tile-sort binning (tile_sort = true): the pairs go straight to their tile's list (atomic
   // cursors) and every list is sorted by (depth, item) on its own; the buffers of the item
   // depth sort, the row-span table and the second key / value buffers are then not allocated.
-  //   stage_ell   float4 [KN][2]: ellipse of each live item, in its projection block's segment
+  //   stage_ell   float4 [KN][2]: ellipse of each live item, in its projection block's segment of
+  //              survivors of the cull (surv_blocks u32 [n_proj_groups]: their number)
   //   stage_meta  uint4 [KN]: its depth key, item id, rectangle x0|x1<<16, y0|y1<<16
-  //   (its tiles emitted: sorted_counts)
+  //   (every survivor's tiles emitted, 0 when it is not live: sorted_counts)
   //   block_pairs u32 [n_proj_groups], super_pairs u64, super_live u32 [ceil(n_proj_groups / 256)]:
   //              pairs of each projection block's live items; pairs and live items of 256 blocks
   //   tile_cursor u32 [kTileSubLists][n_tiles][kCursorStride]: next free pair of each tile's
@@ -137,7 +139,7 @@ struct Layout {
   int sorted;               // buffer (keys[], vals[]) holding the sorted pairs
   size_t zero_bytes;        // the buffers from `status` on that start at zero, cleared together
   int scan_slabs;           // blocks per view of the tile scan (kScanRows tile rows each)
-  size_t stage_ell, stage_meta, block_pairs, super_pairs, super_live, tile_cursor, long_tiles;
+  size_t stage_ell, stage_meta, surv_blocks, block_pairs, super_pairs, super_live, tile_cursor, long_tiles;
   size_t total;
 };
 

@@ -110,6 +110,32 @@ __device__ __forceinline__ uint32_t pack16(int lo, int hi) {
   return static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
 }
 
+// Attribute loads with the storage types known at compile time: DT the attributes' gs_dtype_t, MF32 whether
+// the means are FP32 (else their type is looked up per load).
+template <int DT>
+__device__ __forceinline__ float ld_attr(const void* p, int64_t i) {
+  return load_attr(p, i, DT);
+}
+template <bool MF32>
+__device__ __forceinline__ float ld_mean(const GaussPtrs& G, int64_t i) {
+  return MF32 ? load_attr(G.means, i, GS_F32) : load_attr(G.means, i, G.means_dtype);
+}
+
+// A view's camera with the limits of x/z and y/z, in the exact operation order of the projection.
+struct CamLim {
+  gs_camera_t cam;
+  float limx, limy;
+};
+// Its camera (read through one pointer, so that its 16 numbers don't have to stay in registers).
+struct CamRef {
+  const gs_camera_t* cam;
+  float limx, limy;
+};
+__device__ __forceinline__ CamLim cam_lim(const Layout& L, const gs_camera_t& cam) {
+  return {cam, __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, static_cast<float>(L.W)), cam.fx)),
+          __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, static_cast<float>(L.H)), cam.fy))};
+}
+
 // Whether an item in front of the near plane certainly has an empty tile rectangle, from a
 // bound on its radius that needs no covariance: each row of R Q S (R, Q rotations, S the
 // scales) has length <= max S, so |m1| <= (fx / z)(1 + |tx|) max S (m1, m2: the rows of J R Q S
@@ -124,15 +150,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ bool off_screen(const Layout& L, const gs_camera_t& cam, float xc, float yc, float zc,
+__device__ __forceinline__ bool off_screen(const Layout& L, const CamRef& C, float xc, float yc, float zc,
                                            const float (&ls)[3]) {
+  const gs_camera_t& cam = *C.cam;
   const float smax = __expf(fmaxf(ls[0], fmaxf(ls[1], ls[2]))) * 1.002f;
   const float iz = __fdividef(1.0f, zc);
   const float xz = xc * iz, yz = yc * iz;
-  const float limx = 1.3f * __fdividef(0.5f * static_cast<float>(L.W), cam.fx);
-  const float limy = 1.3f * __fdividef(0.5f * static_cast<float>(L.H), cam.fy);
-  const float m1 = fabsf(cam.fx) * iz * (1.0f + fminf(fabsf(xz), limx)) * smax;
-  const float m2 = fabsf(cam.fy) * iz * (1.0f + fminf(fabsf(yz), limy)) * smax;
+  const float m1 = fabsf(cam.fx) * iz * (1.0f + fminf(fabsf(xz), C.limx)) * smax;
+  const float m2 = fabsf(cam.fy) * iz * (1.0f + fminf(fabsf(yz), C.limy)) * smax;
   const float rb = 3.0f * sqrt_approx(m1 * m1 + m2 * m2 + 1.0f) * 1.01f + 2.0f;
   const float u = cam.fx * xz + cam.cx, v = cam.fy * yz + cam.cy;
   const float mu = 1e-4f * fabsf(u) + 1.0f, mv = 1e-4f * fabsf(v) + 1.0f;
@@ -150,16 +175,20 @@ struct Projected {
   bool live;  // has an ellipse and a non-empty rectangle: its rows are examined next
 };
 
-__device__ __forceinline__ Projected project_item(const Layout& L, const GaussPtrs& G, const gs_camera_t& cam,
-                                                  int64_t idx, int64_t g, uint8_t* __restrict__ ws) {
+template <int DT, bool MF32>
+__device__ __forceinline__ Projected project_item(const Layout& L, const GaussPtrs& G, const CamRef& C, int64_t idx,
+                                                  int64_t g, uint8_t* __restrict__ ws) {
   Projected P{};
-  const float p0 = load_attr(G.means, 3 * g + 0, G.means_dtype);
-  const float p1 = load_attr(G.means, 3 * g + 1, G.means_dtype);
-  const float p2 = load_attr(G.means, 3 * g + 2, G.means_dtype);
+  const gs_camera_t& cam = *C.cam;
+  const float p0 = ld_mean<MF32>(G, 3 * g + 0);
+  const float p1 = ld_mean<MF32>(G, 3 * g + 1);
+  const float p2 = ld_mean<MF32>(G, 3 * g + 2);
   float ls[3], q[4];
-  for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, G.dtype);
-  for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, G.dtype);
-  const float lg = load_attr(G.logits, g, G.dtype);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) ls[j] = ld_attr<DT>(G.log_scales, 3 * g + j);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) q[j] = ld_attr<DT>(G.quats, 4 * g + j);
+  const float lg = ld_attr<DT>(G.logits, g);
   const float* R = cam.R;
   const float* t = cam.t;
   // ---------------- discrete path: fixed binary32 operation order -----------------
@@ -200,8 +229,7 @@ __device__ __forceinline__ Projected project_item(const Layout& L, const GaussPt
     for (int j = 0; j < 3; ++j)
       Nm[i][j] = __fmaf_rn(R[3 * i + 0], M[0][j], __fmaf_rn(R[3 * i + 1], M[1][j], __fmul_rn(R[3 * i + 2], M[2][j])));
   const float xz_ = __fdiv_rn(xc, zc), yz_ = __fdiv_rn(yc, zc);
-  const float limx = __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, static_cast<float>(L.W)), cam.fx));
-  const float limy = __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, static_cast<float>(L.H)), cam.fy));
+  const float limx = C.limx, limy = C.limy;
   const float txz = fminf(fmaxf(xz_, -limx), limx);
   const float tyz = fminf(fmaxf(yz_, -limy), limy);
   const float j00 = __fdiv_rn(cam.fx, zc), j02 = -__fmul_rn(j00, txz);
@@ -287,9 +315,8 @@ __device__ __forceinline__ Projected project_item(const Layout& L, const GaussPt
 // live_mask, its binning record (depth key, tiles emitted, item id, row-span entries) to the
 // block's segment of the staging arrays in item order (compacted by k_live_copy), its depth
 // key's digits to the item-sort histograms. The last block to finish scans the blocks' live
-// counts into their first positions among the live items. For the tile-sort binning
-// (L.tile_sort) the record holds the ellipse and rectangle instead, pass 2 and the histograms
-// are left out, and the tile scan and the emission do the rest.
+// counts into their first positions among the live items. (For the tile-sort binning see
+// k_project_tiles.)
 // The block of items (in item order) that launched block b takes. The n blocks of items are seen
 // as rows of Bv = ceil(n / K) blocks, one row per view (rows cut at block boundaries, so a row
 // is about one view's items; the last row may be shorter), and the launch order walks this
@@ -314,83 +341,110 @@ __device__ __forceinline__ int64_t proj_block(const Layout& L, int64_t b) {
   return k * bv + r;
 }
 
-// (Compiled for 4 resident blocks per SM, 64 registers: the kernel is latency-bound, and 32
-// warps per SM hide more of it than 24; 12% faster at aerial2m than at 3 blocks.)
-__global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
-                                                         uint8_t* __restrict__ ws) {
-  pdl_wait();
-  constexpr int kWords = kProjItemsMax / 32;
-  static_assert(kWords == 64, "the survivor scan below gives each lane of warp 0 two mask words");
-  static_assert(kWords % (kProjThreads / 32) == 0, "phase 1 covers the mask words in whole rounds");
-  const int words = L.proj_items / 32;
-  const int64_t blk = proj_block(L, blockIdx.x);
-  const int64_t first = blk * L.proj_items;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  __shared__ uint32_t s_hist[4 * 256];
-  // the block's rectangles are first added into a shared copy of its first view's difference
-  // grid (when it fits), then flushed with one global atomic per non-zero cell
-  __shared__ int32_t s_grid[kProjGridCells];
-  __shared__ uint32_t s_surv[kWords], s_spre[kWords + 1], s_live[kWords];
-  __shared__ uint32_t s_wcnt[kProjThreads / 32];
-  __shared__ uint32_t s_wpairs[kProjThreads / 32];
-  __shared__ uint32_t s_seg, s_pairs;  // the block's live items so far and their pairs
-  __shared__ int s_acc[kProjThreads / 32][3][32];  // per warp and lane: tiles, first row, last row
-  __shared__ int s_carry[kProjThreads / 32][32];   // tiles of an item's rows already written
-  __shared__ uint8_t s_owner[kProjThreads / 32][32];  // the lanes whose items own rows, in order
-  // the first kSpanCache row spans of each warp's round (pass 1), read again by pass 2
-  __shared__ int2 s_span[kProjThreads / 32][kSpanCache];
-  const int gstride = L.Tx + 1;
-  const int gcells = gstride * (L.Ty + 1);
-  const bool use_sgrid = gcells <= kProjGridCells;
-  const int copy = static_cast<int>(blk & (L.diff_copies - 1));  // the block's copy of the span grids
-  const int k_block = static_cast<int>(first / (L.N > 0 ? L.N : 1));
-  if (!L.tile_sort)
-    for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads) s_hist[i] = 0;
-  if (threadIdx.x < kWords) s_live[threadIdx.x] = 0;
-  if (threadIdx.x == 0) s_seg = s_pairs = 0;
+// Whether all four are finite: x 0 is 0 for a finite x, else not a number.
+__device__ __forceinline__ bool all_finite(float a, float b, float c, float d) {
+  return __fmaf_rn(a, 0.0f, __fmaf_rn(b, 0.0f, __fmaf_rn(c, 0.0f, __fmul_rn(d, 0.0f)))) == 0.0f;
+}
+__device__ __forceinline__ void clear_grid(int32_t* s_grid, int cells) {
+  for (int i = threadIdx.x; 4 * i < cells; i += kProjThreads) reinterpret_cast<int4*>(s_grid)[i] = make_int4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void flush_grid(const int32_t* s_grid, int cells, int32_t* __restrict__ grid) {
+  for (int i = threadIdx.x; 4 * i < cells; i += kProjThreads) {
+    const int4 v = reinterpret_cast<const int4*>(s_grid)[i];
+    if (v.x) atomicAdd(&grid[4 * i], v.x);
+    if (v.y) atomicAdd(&grid[4 * i + 1], v.y);
+    if (v.z) atomicAdd(&grid[4 * i + 2], v.z);
+    if (v.w) atomicAdd(&grid[4 * i + 3], v.w);
+  }
+}
+static_assert(kProjGridCells % 4 == 0, "the span grid is cleared and flushed four cells at a time");
 
-  // ---------------- phase 1: every item --------------------------------------------
-  for (int r = 0; r < kWords / (kProjThreads / 32); ++r) {
+// What the two phases share. The cameras of up to kProjViews views from the block's first one on; a
+// block that spans more (few Gaussians, many views) reads the others from global memory.
+constexpr int kProjWords = kProjItemsMax / 32;
+struct ProjShared {
+  CamLim cam[kProjViews];
+  uint32_t surv[kProjWords], spre[kProjWords + 1], live[kProjWords];
+  uint16_t list[kProjItemsMax];  // the survivors' item numbers in the block, in item order
+};
+
+// View and Gaussian of item first + li; rem0: the Gaussian of the block's first item (32-bit arithmetic:
+// K N < 2^31, and a division only in a block that crosses into another view).
+struct ItemId {
+  int kk;  // views after the block's first
+  uint32_t g;
+};
+__device__ __forceinline__ ItemId item_id(uint32_t rem0, uint32_t li, uint32_t N) {
+  const uint32_t r = rem0 + li;
+  if (r < N) return {0, r};
+  const uint32_t q = r / N;
+  return {static_cast<int>(q), r - q * N};
+}
+__device__ __forceinline__ CamRef item_cam(const Layout& L, const ProjShared& C, const gs_camera_t* __restrict__ cams,
+                                           int k_block, int kk) {
+  if (kk < kProjViews) return {&C.cam[kk].cam, C.cam[kk].limx, C.cam[kk].limy};
+  const gs_camera_t& cam = cams[k_block + kk];
+  const CamLim c = cam_lim(L, cam);
+  return {&cam, c.limx, c.limy};
+}
+
+// Phase 1. Returns the number of survivors, listed in C.list; C.live is cleared. Ends with a barrier.
+template <int DT, bool MF32>
+__device__ __forceinline__ int cull_items(const Layout& L, const GaussPtrs& G, const gs_camera_t* __restrict__ cams,
+                                          uint8_t* __restrict__ ws, int64_t first, int k_block, uint32_t rem0,
+                                          ProjShared& C) {
+  static_assert(kProjWords == 64, "the survivor scan below gives each lane of warp 0 two mask words");
+  constexpr int kWarps = kProjThreads / 32;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const uint32_t N = static_cast<uint32_t>(L.N), left = static_cast<uint32_t>(L.KN - first);
+  if (threadIdx.x < kProjViews && k_block + static_cast<int>(threadIdx.x) < L.K)
+    C.cam[threadIdx.x] = cam_lim(L, cams[k_block + threadIdx.x]);
+  if (threadIdx.x < kProjWords) C.live[threadIdx.x] = 0;
+  __syncthreads();
+  for (int r = 0; r < kProjWords / kWarps; ++r) {
     if (r * kProjThreads >= L.proj_items) {  // (block-uniform) the block's mask words end here
-      if (lane == 0) s_surv[r * (kProjThreads / 32) + wib] = 0u;
+      if (lane == 0) C.surv[r * kWarps + wib] = 0u;
       continue;
     }
-    const int64_t idx = first + r * kProjThreads + threadIdx.x;
+    const uint32_t li = r * kProjThreads + threadIdx.x;
     bool surv = false;
-    if (idx < L.KN) {
-      const int k = static_cast<int>(idx / L.N);
-      const int64_t g = idx - static_cast<int64_t>(k) * L.N;
-      const gs_camera_t& cam = cams[k];
-      const float p0 = load_attr(G.means, 3 * g + 0, G.means_dtype);
-      const float p1 = load_attr(G.means, 3 * g + 1, G.means_dtype);
-      const float p2 = load_attr(G.means, 3 * g + 2, G.means_dtype);
+    if (li < left) {
+      const ItemId id = item_id(rem0, li, N);
+      const int k = k_block + id.kk;
+      const int64_t g = id.g;
+      const CamRef cl = item_cam(L, C, cams, k_block, id.kk);
+      const gs_camera_t& cam = *cl.cam;
+      const float p0 = ld_mean<MF32>(G, 3 * g + 0);
+      const float p1 = ld_mean<MF32>(G, 3 * g + 1);
+      const float p2 = ld_mean<MF32>(G, 3 * g + 2);
       float ls[3];
-      for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, G.dtype);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) ls[j] = ld_attr<DT>(G.log_scales, 3 * g + j);
       // colour and opacity: once per Gaussian, or per item when the colour depends on the view
       if (k == 0 || L.color_stride != 0) {
         float q[4];
-        for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, G.dtype);
-        const float lg = load_attr(G.logits, g, G.dtype);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = ld_attr<DT>(G.quats, 4 * g + j);
+        const float lg = ld_attr<DT>(G.logits, g);
         float c0, c1, c2;
         bool finite_c = true;
         if (L.color_mode == GS_COLOR_SH) {
           const ShDir u = sh_dir(p0, p1, p2, cam);
           float Y[kShMaxCoeffs];
           sh_basis(u.x, u.y, u.z, Y);
-          const float3 raw = sh_raw(G.rgb, G.dtype, g, L.sh_coeffs, Y, finite_c);
+          const float3 raw = sh_raw(G.rgb, DT, g, L.sh_coeffs, Y, finite_c);
           c0 = fmaxf(raw.x, 0.0f), c1 = fmaxf(raw.y, 0.0f), c2 = fmaxf(raw.z, 0.0f);
         } else {
-          c0 = load_attr(G.rgb, 3 * g + 0, G.dtype);
-          c1 = load_attr(G.rgb, 3 * g + 1, G.dtype);
-          c2 = load_attr(G.rgb, 3 * g + 2, G.dtype);
-          finite_c = isfinite(c0) && isfinite(c1) && isfinite(c2);
+          c0 = ld_attr<DT>(G.rgb, 3 * g + 0);
+          c1 = ld_attr<DT>(G.rgb, 3 * g + 1);
+          c2 = ld_attr<DT>(G.rgb, 3 * g + 2);
+          finite_c = all_finite(0.0f, c0, c1, c2);
         }
         const float o = 1.0f / (1.0f + expf(-lg));
         at<float4>(ws, L.color_opacity)[k * L.color_stride + g] = make_float4(c0, c1, c2, o);
-        const bool finite = isfinite(p0) && isfinite(p1) && isfinite(p2) && isfinite(ls[0]) && isfinite(ls[1]) &&
-                            isfinite(ls[2]) && isfinite(q[0]) && isfinite(q[1]) && isfinite(q[2]) && isfinite(q[3]) &&
-                            isfinite(lg) && finite_c;
-        if (k == 0 && !finite) atomicOr(&at<Status>(ws, L.status)->err, GS_DEVERR_NONFINITE);
+        if (k == 0 && !(finite_c && all_finite(lg, p0, p1, p2) && all_finite(q[0], ls[0], ls[1], ls[2]) &&
+                        all_finite(0.0f, q[1], q[2], q[3])))
+          atomicOr(&at<Status>(ws, L.status)->err, GS_DEVERR_NONFINITE);
       }
       const float* R = cam.R;
       const float* t = cam.t;
@@ -399,31 +453,66 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
       const float xc = __fmaf_rn(R[0], p0, __fmaf_rn(R[1], p1, __fmaf_rn(R[2], p2, t[0])));
       const float yc = __fmaf_rn(R[3], p0, __fmaf_rn(R[4], p1, __fmaf_rn(R[5], p2, t[1])));
       const float zc = __fmaf_rn(R[6], p0, __fmaf_rn(R[7], p1, __fmaf_rn(R[8], p2, t[2])));
-      surv = zc > L.near_plane && !off_screen(L, cam, xc, yc, zc, ls);
+      surv = zc > L.near_plane && !off_screen(L, cl, xc, yc, zc, ls);
     }
     const uint32_t ballot = __ballot_sync(0xffffffffu, surv);
-    if (lane == 0) s_surv[r * (kProjThreads / 32) + wib] = ballot;
+    if (lane == 0) C.surv[r * kWarps + wib] = ballot;
   }
   __syncthreads();
-  // exclusive prefix of the survivors over the mask words (warp 0; kWords = 2 per lane)
+  // exclusive prefix of the survivors over the mask words (warp 0; two words per lane)
   if (wib == 0) {
-    const uint32_t c0 = __popc(s_surv[2 * lane]), c1 = __popc(s_surv[2 * lane + 1]);
+    const uint32_t c0 = __popc(C.surv[2 * lane]), c1 = __popc(C.surv[2 * lane + 1]);
     uint32_t incl = c0 + c1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
-    s_spre[2 * lane] = incl - c0 - c1;
-    s_spre[2 * lane + 1] = incl - c1;
-    if (lane == 31) s_spre[kWords] = incl;
+    C.spre[2 * lane] = incl - c0 - c1;
+    C.spre[2 * lane + 1] = incl - c1;
+    if (lane == 31) C.spre[kProjWords] = incl;
   }
   __syncthreads();
-  const int n_surv = static_cast<int>(s_spre[kWords]);
-  if (use_sgrid && n_surv > 0) {
-    for (int i = threadIdx.x; i < gcells; i += kProjThreads) s_grid[i] = 0;
+  for (int w = wib; w * 32 < L.proj_items; w += kWarps) {
+    const uint32_t word = C.surv[w];
+    if ((word >> lane) & 1u)
+      C.list[C.spre[w] + __popc(word & ((1u << lane) - 1u))] = static_cast<uint16_t>(32 * w + lane);
   }
   __syncthreads();
+  return static_cast<int>(C.spre[kProjWords]);
+}
+
+// (Compiled for 4 resident blocks per SM, 64 registers: the kernel is latency-bound, and 32
+// warps per SM hide more of it than 24; 12% faster at 16 aerial views of 2M Gaussians than at 3 blocks.)
+template <int DT, bool MF32>
+__global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
+                                                         uint8_t* __restrict__ ws) {
+  pdl_wait();
+  const int words = L.proj_items / 32;
+  const int64_t blk = proj_block(L, blockIdx.x);
+  const int64_t first = blk * L.proj_items;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  __shared__ uint32_t s_hist[4 * 256];
+  // the block's rectangles are first added into a shared copy of its first view's difference
+  // grid (when it fits), then flushed with one global atomic per non-zero cell
+  __shared__ __align__(16) int32_t s_grid[kProjGridCells];
+  __shared__ ProjShared C;
+  __shared__ uint32_t s_wcnt[kProjThreads / 32];
+  __shared__ uint32_t s_seg;  // the block's live items so far
+  __shared__ int s_acc[kProjThreads / 32][3][32];  // per warp and lane: tiles, first row, last row
+  __shared__ int s_carry[kProjThreads / 32][32];   // tiles of an item's rows already written
+  __shared__ uint8_t s_owner[kProjThreads / 32][32];  // the lanes whose items own rows, in order
+  // the first kSpanCache row spans of each warp's round (pass 1), read again by pass 2
+  __shared__ int2 s_span[kProjThreads / 32][kSpanCache];
+  const int gstride = L.Tx + 1;
+  const int gcells = gstride * (L.Ty + 1);
+  const bool use_sgrid = gcells <= kProjGridCells;
+  const int k_block = static_cast<int>(static_cast<uint32_t>(first) / static_cast<uint32_t>(L.N > 0 ? L.N : 1));
+  const uint32_t rem0 = static_cast<uint32_t>(first - static_cast<int64_t>(k_block) * L.N);
+  for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads) s_hist[i] = 0;
+  if (use_sgrid) clear_grid(s_grid, gcells);
+  if (threadIdx.x == 0) s_seg = 0;
+  const int n_surv = cull_items<DT, MF32>(L, G, cams, ws, first, k_block, rem0, C);
 
   // ---------------- phase 2: the survivors, kProjThreads per round ---------------------
   uint32_t lm;
@@ -434,16 +523,12 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
     int kv = 0;
     Projected P{};
     if (j < n_surv) {
-      // the j-th survivor: its mask word (binary search over the prefix), then its bit
-      int lo = 0, hi = kWords;  // s_spre[lo] <= j < s_spre[hi]
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (s_spre[mid] <= static_cast<uint32_t>(j)) lo = mid; else hi = mid;
-      }
-      const int bit = __fns(s_surv[lo], 0, j - static_cast<int>(s_spre[lo]) + 1);
-      idx = first + 32 * lo + bit;
-      kv = static_cast<int>(idx / L.N);
-      P = project_item(L, G, cams[kv], idx, idx - static_cast<int64_t>(kv) * L.N, ws);
+      const uint32_t li = C.list[j];
+      const ItemId id = item_id(rem0, li, static_cast<uint32_t>(L.N));
+      idx = first + li;
+      kv = k_block + id.kk;
+      const CamRef cl = item_cam(L, C, cams, k_block, id.kk);
+      P = project_item<DT, MF32>(L, G, cl, idx, id.g, ws);
     }
     // the rectangles' rows, shared out over the warp: the warp's items' rows are numbered
     // consecutively (item by item) and examined 32 at a time, one row per lane, so a warp
@@ -480,7 +565,7 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
             atomicMax(&s_acc[wib][2][o], ty);
             int32_t* dg = (use_sgrid && ok == k_block)
                               ? s_grid
-                              : at<int32_t>(ws, L.tile_diff) + (static_cast<int64_t>(ok) * L.diff_copies + copy) * gcells;
+                              : at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(ok) * gcells;
             atomicAdd(&dg[ty * gstride + sp.x], 1);  // row-wise prefix sum: pairs per tile
             atomicAdd(&dg[ty * gstride + sp.y + 1], -1);
           }
@@ -499,10 +584,9 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
       at<uint32_t>(ws, L.proj_depth_key)[idx] = item_key;
       at<int32_t>(ws, L.proj_radius)[idx] = P.radius;
     }
-    // row-span table entries for the item's rows first..last (one counter atomic per warp); the
-    // tile-sort binning computes the spans again from the staged ellipse instead
+    // row-span table entries for the item's rows first..last (one counter atomic per warp)
     uint2 rows_out = make_uint2(0, 0);
-    if (!L.tile_sort) {
+    {
       uint32_t incl = nrows;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -567,70 +651,38 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
     // the live items of this round, in item order: their bits, and their binning records at
     // the end of the block's segment
     const uint32_t ballot = __ballot_sync(0xffffffffu, is_live);
-    const uint32_t wpairs = __reduce_add_sync(0xffffffffu, is_live ? count : 0u);
-    if (lane == 0) {
-      s_wcnt[wib] = __popc(ballot);
-      s_wpairs[wib] = wpairs;
-    }
+    if (lane == 0) s_wcnt[wib] = __popc(ballot);
     __syncthreads();
-    // (the round's totals are read between the barriers: the next round overwrites the warps' counts)
-    uint32_t before = s_seg, round_live = 0, round_pairs = 0;
+    // (the round's total is read between the barriers: the next round overwrites the warps' counts)
+    uint32_t before = s_seg, round_live = 0;
 #pragma unroll
     for (int w = 0; w < kProjThreads / 32; ++w) {
       const uint32_t c = s_wcnt[w];
       before += w < wib ? c : 0u;
       round_live += c;
-      round_pairs += s_wpairs[w];
     }
     if (is_live) {
-      atomicOr(&s_live[(idx - first) >> 5], 1u << (idx & 31));
+      atomicOr(&C.live[(idx - first) >> 5], 1u << (idx & 31));
       const int64_t pos = first + before + __popc(ballot & lm);
       at<uint32_t>(ws, L.sorted_counts)[pos] = count;          // staging: tiles emitted
-      if (L.tile_sort) {
-        const Ellipse& E = P.E;
-        at<float4>(ws, L.stage_ell)[2 * pos] = make_float4(E.u, E.v, E.b, E.inv_c);
-        at<float4>(ws, L.stage_ell)[2 * pos + 1] = make_float4(E.sdet, E.hx, E.hy, E.kxy);
-        at<uint4>(ws, L.stage_meta)[pos] =
-            make_uint4(item_key, static_cast<uint32_t>(idx), pack16(P.x0, P.x1), pack16(P.y0, P.y1));
-      } else {
-        at<uint32_t>(ws, L.item_keys[1])[pos] = item_key;        // staging: depth-sort key
-        at<uint32_t>(ws, L.item_vals[1])[pos] = static_cast<uint32_t>(idx);  // staging: item id
-        at<uint2>(ws, L.item_rect)[pos] = rows_out;              // staging: row-span entries (as uint2)
+      at<uint32_t>(ws, L.item_keys[1])[pos] = item_key;        // staging: depth-sort key
+      at<uint32_t>(ws, L.item_vals[1])[pos] = static_cast<uint32_t>(idx);  // staging: item id
+      at<uint2>(ws, L.item_rect)[pos] = rows_out;              // staging: row-span entries (as uint2)
 #pragma unroll
-        for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p * 256 + ((item_key >> (8 * p)) & 0xffu)], 1u);
-      }
+      for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p * 256 + ((item_key >> (8 * p)) & 0xffu)], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      s_seg += round_live;
-      s_pairs += round_pairs;
-    }
+    if (threadIdx.x == 0) s_seg += round_live;
   }
   __syncthreads();
   // the block's live mask words, its live count, its span grid and its histograms
   if (threadIdx.x < words) {
     const int64_t w = first / 32 + threadIdx.x;
-    if (w < (L.KN + 31) / 32) at<uint32_t>(ws, L.live_mask)[w] = s_live[threadIdx.x];
+    if (w < (L.KN + 31) / 32) at<uint32_t>(ws, L.live_mask)[w] = C.live[threadIdx.x];
   }
   if (threadIdx.x == 0) at<uint32_t>(ws, L.live_blocks)[blk] = s_seg;
-  if (use_sgrid && n_surv > 0 && k_block < L.K) {
-    int32_t* dg = at<int32_t>(ws, L.tile_diff) + (static_cast<int64_t>(k_block) * L.diff_copies + copy) * gcells;
-    for (int i = threadIdx.x; i < gcells; i += kProjThreads)
-      if (s_grid[i]) atomicAdd(&dg[i], s_grid[i]);
-  }
-  if (L.tile_sort) {  // the emission finds the blocks' first positions; the item sort does not run
-    if (threadIdx.x == 0) {
-      at<uint32_t>(ws, L.block_pairs)[blk] = s_pairs;
-      if (s_pairs) {
-        using u64 = unsigned long long;
-        atomicAdd(reinterpret_cast<u64*>(at<uint64_t>(ws, L.super_pairs) + blk / 256), static_cast<u64>(s_pairs));
-        atomicAdd(at<uint32_t>(ws, L.super_live) + blk / 256, s_seg);
-        atomicAdd(reinterpret_cast<u64*>(&at<Status>(ws, L.status)->total_pairs), static_cast<u64>(s_pairs));
-      }
-    }
-    pdl_trigger();
-    return;
-  }
+  if (use_sgrid && n_surv > 0 && k_block < L.K)
+    flush_grid(s_grid, gcells, at<int32_t>(ws, L.tile_diff) + static_cast<int64_t>(k_block) * gcells);
   uint32_t* hist = at<uint32_t>(ws, L.item_hist);
   for (int i = threadIdx.x; i < 4 * 256; i += kProjThreads)
     if (s_hist[i]) atomicAdd(&hist[i], s_hist[i]);
@@ -682,6 +734,126 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
   pdl_trigger();
 }
 
+// The projection for the tile-sort binning. Phase 2 needs no barriers: a warp takes 32 survivors at a time
+// and stages each survivor's binning record (tiles emitted, and for a live one the ellipse, depth key and
+// rectangle) at its place among the block's survivors; the emission leaves the dead ones out. One row
+// pass: it counts each item's emitted tiles and adds the spans to the block's copy of the span grid.
+// Bound by instruction issue (52..66% of the slots) and, at 28 of 64 warps, latency. Storage types fixed
+// at compile time, cameras in shared memory, survivors listed instead of searched for, and no barrier
+// per 256 survivors: 2 views of 1M Gaussians 110 -> 87 us, 8 of 250k 107 -> 86, 2 of 100k 28 -> 25
+// (device time of the kernel alone). 3 blocks per SM without the 64-register limit 100 us, 5 blocks
+// with spills 82 / 88; blocks of half the items 92 / 96 (clearing and flushing the grid).
+template <int DT, bool MF32>
+__global__ void __launch_bounds__(kProjThreads, 4)
+    k_project_tiles(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams, uint8_t* __restrict__ ws) {
+  pdl_wait();
+  constexpr int kWarps = kProjThreads / 32;
+  const int words = L.proj_items / 32;
+  const int64_t blk = proj_block(L, blockIdx.x);
+  const int64_t first = blk * L.proj_items;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  __shared__ __align__(16) int32_t s_grid[kProjGridCells];
+  __shared__ ProjShared C;
+  __shared__ int s_count[kWarps][32];        // tiles emitted by each lane's item
+  __shared__ uint8_t s_owner[kWarps][32];    // the lanes whose items own rows, in order
+  __shared__ uint32_t s_pairs, s_nlive;
+  const int gstride = L.Tx + 1;
+  const int gcells = gstride * (L.Ty + 1);
+  const bool use_sgrid = gcells <= kProjGridCells;
+  const int64_t copy = blk & (L.diff_copies - 1);  // the block's copy of the span grids
+  const int k_block = static_cast<int>(static_cast<uint32_t>(first) / static_cast<uint32_t>(L.N));
+  const uint32_t rem0 = static_cast<uint32_t>(first - static_cast<int64_t>(k_block) * L.N);
+  if (use_sgrid) clear_grid(s_grid, gcells);
+  if (threadIdx.x == 0) s_pairs = s_nlive = 0;
+  const int n_surv = cull_items<DT, MF32>(L, G, cams, ws, first, k_block, rem0, C);
+
+  uint32_t pairs = 0;
+  for (int base = wib * 32; base < n_surv; base += kProjThreads) {
+    const int j = base + lane;
+    int64_t idx = -1;
+    int kk = 0;
+    uint32_t li = 0;
+    Projected P{};
+    if (j < n_surv) {
+      li = C.list[j];
+      const ItemId id = item_id(rem0, li, static_cast<uint32_t>(L.N));
+      idx = first + li;
+      kk = id.kk;
+      const CamRef cl = item_cam(L, C, cams, k_block, id.kk);
+      P = project_item<DT, MF32>(L, G, cl, idx, id.g, ws);
+    }
+    // the rectangles' rows, shared out over the warp: the warp's items' rows are numbered
+    // consecutively (item by item) and examined 32 at a time, one row per lane
+    int2 rows = make_int2(0, 0);
+    if (P.live) rows = ellipse_rows(P.E, P.y0, P.y1);
+    const bool any = rows.y > rows.x;
+    const uint32_t owners = __ballot_sync(0xffffffffu, any);
+    __syncwarp();
+    if (any) s_owner[wib][__popc(owners & ((1u << lane) - 1u))] = static_cast<uint8_t>(lane);
+    s_count[wib][lane] = 0;
+    __syncwarp();
+    int total;
+    const int st = warp_exclusive_scan(rows.y - rows.x, total);
+    for (int rb = 0; rb < total; rb += 32) {
+      const int r = rb + lane;
+      const int o = s_owner[wib][warp_owner_rank(st, any, rb)];
+      const Ellipse eo = shfl_ellipse(P.E, o);
+      const int ox0 = __shfl_sync(0xffffffffu, P.x0, o), ox1 = __shfl_sync(0xffffffffu, P.x1, o);
+      const int ty = __shfl_sync(0xffffffffu, rows.x - st, o) + r;
+      const int okk = __shfl_sync(0xffffffffu, kk, o);
+      if (r < total) {
+        const int2 sp = row_span(eo, ty, ox0, ox1);
+        if (sp.x <= sp.y) {
+          atomicAdd(&s_count[wib][o], sp.y - sp.x + 1);
+          int32_t* dg = (use_sgrid && okk == 0)
+                            ? s_grid
+                            : at<int32_t>(ws, L.tile_diff) + ((k_block + okk) * static_cast<int64_t>(L.diff_copies) + copy) * gcells;
+          atomicAdd(&dg[ty * gstride + sp.x], 1);  // row-wise prefix sum: pairs per tile
+          atomicAdd(&dg[ty * gstride + sp.y + 1], -1);
+        }
+      }
+    }
+    __syncwarp();
+    const uint32_t count = static_cast<uint32_t>(s_count[wib][lane]);
+    if (idx >= 0) at<uint32_t>(ws, L.sorted_counts)[first + j] = count;
+    if (count > 0) {
+      const Ellipse& E = P.E;
+      const uint32_t key = __float_as_uint(P.z), rx = pack16(P.x0, P.x1), ry = pack16(P.y0, P.y1);
+      at<float4>(ws, L.stage_ell)[2 * (first + j)] = make_float4(E.u, E.v, E.b, E.inv_c);
+      at<float4>(ws, L.stage_ell)[2 * (first + j) + 1] = make_float4(E.sdet, E.hx, E.hy, E.kxy);
+      at<uint4>(ws, L.stage_meta)[first + j] = make_uint4(key, static_cast<uint32_t>(idx), rx, ry);
+      at<int4>(ws, L.proj_tiles)[idx] = make_int4(0, static_cast<int>(rx), static_cast<int>(ry), static_cast<int>(count));
+      at<uint32_t>(ws, L.proj_depth_key)[idx] = key;
+      at<int32_t>(ws, L.proj_radius)[idx] = P.radius;
+      atomicOr(&C.live[li >> 5], 1u << (li & 31));
+      pairs += count;
+    }
+    const uint32_t ballot = __ballot_sync(0xffffffffu, count > 0);
+    if (lane == 0 && ballot) atomicAdd(&s_nlive, static_cast<uint32_t>(__popc(ballot)));
+  }
+  pairs = __reduce_add_sync(0xffffffffu, pairs);
+  if (lane == 0 && pairs) atomicAdd(&s_pairs, pairs);
+  __syncthreads();
+  if (threadIdx.x < words) {
+    const int64_t w = first / 32 + threadIdx.x;
+    if (w < (L.KN + 31) / 32) at<uint32_t>(ws, L.live_mask)[w] = C.live[threadIdx.x];
+  }
+  if (use_sgrid && n_surv > 0)
+    flush_grid(s_grid, gcells, at<int32_t>(ws, L.tile_diff) + (k_block * static_cast<int64_t>(L.diff_copies) + copy) * gcells);
+  if (threadIdx.x == 0) {
+    at<uint32_t>(ws, L.live_blocks)[blk] = s_nlive;
+    at<uint32_t>(ws, L.surv_blocks)[blk] = static_cast<uint32_t>(n_surv);
+    at<uint32_t>(ws, L.block_pairs)[blk] = s_pairs;
+    if (s_pairs) {
+      using u64 = unsigned long long;
+      atomicAdd(reinterpret_cast<u64*>(at<uint64_t>(ws, L.super_pairs) + blk / 256), static_cast<u64>(s_pairs));
+      atomicAdd(at<uint32_t>(ws, L.super_live) + blk / 256, s_nlive);
+      atomicAdd(reinterpret_cast<u64*>(&at<Status>(ws, L.status)->total_pairs), static_cast<u64>(s_pairs));
+    }
+  }
+  pdl_trigger();
+}
+
 // Compaction of the live items, in increasing item order k N + g: each projection block's
 // segment of staged binning records goes to the block's first position among the live items,
 // as the depth-sort keys (the item sort's input, with values = positions), the items' ids,
@@ -725,7 +897,23 @@ __global__ void __launch_bounds__(kProjThreads) k_live_copy(Layout L, uint8_t* _
 cudaError_t launch_project(const Layout& L, const GaussPtrs& g, const gs_camera_t* cams, void* ws, cudaStream_t s) {
   auto* w = static_cast<uint8_t*>(ws);
   const unsigned groups = static_cast<unsigned>(L.n_proj_groups);
-  launch(k_project, groups, kProjThreads, 0, s, L, g, cams, w);
+  const bool mf32 = g.means_dtype == GS_F32;
+#define GS_PROJ_M(DT, M)                                                                   \
+  if (L.tile_sort) launch(k_project_tiles<DT, M>, groups, kProjThreads, 0, s, L, g, cams, w); \
+  else launch(k_project<DT, M>, groups, kProjThreads, 0, s, L, g, cams, w)
+#define GS_PROJ(DT)      \
+  if (mf32) {            \
+    GS_PROJ_M(DT, true); \
+  } else {               \
+    GS_PROJ_M(DT, false); \
+  }
+  switch (g.dtype) {
+    case GS_F32: GS_PROJ(GS_F32); break;
+    case GS_BF16: GS_PROJ(GS_BF16); break;
+    default: GS_PROJ(GS_F16); break;
+  }
+#undef GS_PROJ
+#undef GS_PROJ_M
   // (the tile-sort binning's emission compacts the live items itself)
   if (!L.tile_sort) launch(k_live_copy, groups, kProjThreads, 0, s, L, w);
   return cudaGetLastError();

@@ -54,8 +54,9 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
   __shared__ uint32_t s_cnt[2][kWarps], s_live[kWarps];
   __shared__ uint64_t s_pairs[kWarps];
   __shared__ uint32_t s_w0;
-  __shared__ uint8_t s_row[kWarps][32];
-  const uint32_t cnt = at<uint32_t>(ws, L.live_blocks)[b];
+  __shared__ uint32_t s_lv[2][kWarps];
+  __shared__ uint8_t s_row[kWarps][32], s_item[kWarps][32];
+  const uint32_t cnt = at<uint32_t>(ws, L.surv_blocks)[b];  // staged survivors, live or not
   const uint64_t cap = static_cast<uint64_t>(L.cap), total_pairs = st->total_pairs;
   const bool overflow = total_pairs > cap;  // every tile's range is empty
   // the block's first live item and first pair: the sums over 256 blocks before it, then over blocks
@@ -128,28 +129,37 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
     const bool valid = lane < static_cast<int>(share) && j < cnt;
     Ellipse E{};
     uint4 meta = make_uint4(0, 0, 0, 0);
-    uint32_t n = 0;
-    if (valid) {
+    const uint32_t n = valid ? at<uint32_t>(ws, L.sorted_counts)[first + j] : 0u;
+    const bool live = n > 0;
+    if (live) {
       const float4 a = at<float4>(ws, L.stage_ell)[2 * (first + j)], c = at<float4>(ws, L.stage_ell)[2 * (first + j) + 1];
       E = Ellipse{a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
       meta = at<uint4>(ws, L.stage_meta)[first + j];
-      n = at<uint32_t>(ws, L.sorted_counts)[first + j];
     }
     int wtotal;
     const uint32_t excl = static_cast<uint32_t>(warp_exclusive_scan(static_cast<int>(n), wtotal));
-    if (lane == 0) s_cnt[buf][wib] = static_cast<uint32_t>(wtotal);
+    const uint32_t lives = __ballot_sync(0xffffffffu, live), rank = __popc(lives & ((1u << lane) - 1u));
+    if (lane == 0) {
+      s_cnt[buf][wib] = static_cast<uint32_t>(wtotal);
+      s_lv[buf][wib] = __popc(lives);
+    }
     __syncthreads();
-    uint64_t wbase = pairs;  // the warp's first pair
+    uint64_t wbase = pairs;  // the warp's first pair and first live item
+    uint32_t lbase = base;
+#pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-      wbase += w < wib ? s_cnt[buf][w] : 0u;
-      pairs += s_cnt[buf][w];
+      const uint32_t c = s_cnt[buf][w], l = s_lv[buf][w];
+      wbase += w < wib ? c : 0u;
+      lbase += w < wib ? l : 0u;
+      pairs += c;
+      base += l;
     }
     uint32_t g = 0, tile0 = 0;
-    if (valid) {
+    if (live) {
       const uint64_t off = wbase + excl;
-      at<uint32_t>(ws, L.live_kg)[base + j] = meta.y;
-      at<uint32_t>(ws, L.live_count)[base + j] = n;
-      at<uint32_t>(ws, L.live_off)[base + j] = static_cast<uint32_t>(off < cap ? off : cap);
+      at<uint32_t>(ws, L.live_kg)[lbase + rank] = meta.y;
+      at<uint32_t>(ws, L.live_count)[lbase + rank] = n;
+      at<uint32_t>(ws, L.live_off)[lbase + rank] = static_cast<uint32_t>(off < cap ? off : cap);
       const uint32_t k = meta.y / static_cast<uint32_t>(L.N);
       g = meta.y - k * static_cast<uint32_t>(L.N);
       tile0 = static_cast<uint32_t>(k * per_view);
@@ -157,15 +167,16 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
     if (overflow) continue;
     const int x0 = static_cast<int>(meta.z & 0xffffu), x1 = static_cast<int>(meta.z >> 16);
     int2 rows = make_int2(0, 0);
-    if (valid) rows = ellipse_rows(E, static_cast<int>(meta.w & 0xffffu), static_cast<int>(meta.w >> 16));
+    if (live) rows = ellipse_rows(E, static_cast<int>(meta.w & 0xffffu), static_cast<int>(meta.w >> 16));
     int nrows;
     const int rst = warp_exclusive_scan(rows.y - rows.x, nrows);
-    // (the lanes holding an item come first and every one of them has rows, so the rank is the lane)
-    const bool any_rows = rows.y > rows.x;
+    const bool any_rows = rows.y > rows.x;  // (every live item has rows)
+    if (any_rows) s_item[wib][rank] = static_cast<uint8_t>(lane);
+    __syncwarp();
     uint32_t slot0 = static_cast<uint32_t>(wbase);  // first pair of the next 32 rows (total <= cap < 2^30)
     for (int rb = 0; rb < nrows; rb += 32) {
       const int r = rb + lane;
-      const int o = warp_owner_rank(rst, any_rows, rb);
+      const int o = s_item[wib][warp_owner_rank(rst, any_rows, rb)];
       const Ellipse eo = shfl_ellipse(E, o);
       const int ox0 = __shfl_sync(0xffffffffu, x0, o), ox1 = __shfl_sync(0xffffffffu, x1, o);
       const int ty = __shfl_sync(0xffffffffu, rows.x, o) + (r - __shfl_sync(0xffffffffu, rst, o));

@@ -66,3 +66,11 @@ def test_grids_and_views(W, H, K, n):
     """Just 152 tiles, one row of tiles, view boundaries inside projection blocks, ragged sizes."""
     s = make_scene("window500k", n=n, K=K, W=W, H=H, f=0.8 * min(W, 320))
     _check(s.params(), s.cams, W, H, cap=1 << 18)
+
+
+@pytest.mark.parametrize("W,H,K,n", [(200, 150, 12, 40), (200, 150, 9, 1), (64, 48, 12, 40)])
+def test_many_views_in_a_projection_block(W, H, K, n):
+    """So few Gaussians that a projection block spans more views than it keeps cameras of in shared
+    memory; the last one has too few tiles for the tile-sort binning."""
+    s = make_scene("window500k", n=n, K=K, W=W, H=H, f=0.8 * W)
+    _check(s.params(), s.cams, W, H, cap=1 << 16)
