@@ -230,8 +230,12 @@ __device__ __forceinline__ TileCoord tile_coord(const Layout& L, int64_t tile_g)
 // backward, us at 2 / 4 pixels: 672 tiles 133 / 150, 1200 tiles 160 / 150 and 145 / 123, 4032 tiles 195 /
 // 168); forward only from 4000 (300 tiles 28.6 / 36.8, 1200 55 / 53, 3600 with uneven lists 112 / 127,
 // 4032 60 / 58, 9600 236 / 201).
-int default_px(const Layout& L, bool backward) { return L.n_tiles >= (backward ? 1024 : 4000) ? 4 : 2; }
+// A caller who fixes only one of the two passes gets 2 for the other.
 int pick_px(int requested, int fallback) { return (requested == 1 || requested == 2 || requested == 4) ? requested : fallback; }
+int default_px(const Layout& L, bool backward) {
+  if (pick_px(L.fwd_px, 0) || pick_px(L.bwd_px, 0)) return 2;
+  return L.n_tiles >= (backward ? 1024 : 4000) ? 4 : 2;
+}
 // chunk depth: a power of two in [lo, hi], else the default
 int pick_chunk(int requested, int lo, int hi, int fallback) {
   return (requested >= lo && requested <= hi && (requested & (requested - 1)) == 0) ? requested : fallback;

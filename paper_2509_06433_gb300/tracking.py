@@ -22,7 +22,7 @@ def fuses_backward(r) -> bool:
     (gs_raster_fwd_l1_bwd): only when both use the same pixels per thread (then the results are
     those of the two calls bit for bit), and not when the autotuner found two launches faster
     (``r.fused_compositing``)."""
-    px = lambda v: v if v in (1, 2, 4) else 0  # noqa: E731  (0 = the library's choice, the same for both)
+    px = lambda v: v if v in (1, 2, 4) else 2  # noqa: E731  (both 0: the library's choice, the same for both; one: 2)
     c = r.cfg
     return px(c.fwd_px_per_thread) == px(c.bwd_px_per_thread) and getattr(r, "fused_compositing", True)
 
