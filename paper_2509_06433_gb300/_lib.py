@@ -133,8 +133,14 @@ def load(path: str | None = None) -> ctypes.CDLL:
     return _lib
 
 
+_fns = {}  # entry points looked up so far
+
+
 def call(name, *args):
-    code = getattr(load(), name)(*args)
+    fn = _fns.get(name)
+    if fn is None:
+        fn = _fns[name] = getattr(load(), name)
+    code = fn(*args)
     if code != GS_OK:
         raise GsError(name, code)
     return code
