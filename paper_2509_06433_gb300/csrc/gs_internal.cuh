@@ -25,7 +25,7 @@ constexpr int kSortItems = 15;        // keys per thread per onesweep tile (defa
 constexpr int kSortTileKeys = kSortThreads * kSortItems;
 constexpr int kMaxSortPasses = 8;
 constexpr int kPairGradStride = 12;   // floats per pair gradient record (10 used)
-constexpr int kPoseBlock = 256;       // Gaussians / live items per projection-backward block
+constexpr int kPoseBlock = 128;       // Gaussians / live items per projection-backward block
 // Tile-sort binning (tile_sort.cu): each tile's list sorted by its own block.
 constexpr int kTileSortMinTiles = 152;  // fewer tiles than SMs: the global radix sorts instead
 constexpr int kScanRows = 8;            // tile rows per block of the tile scan
@@ -50,7 +50,6 @@ struct Status {
   uint32_t n_live;          // live items: (view, Gaussian) items that emit at least one pair
   uint32_t view_ctr;        // tile-scan blocks started
   uint32_t proj_done;       // projection blocks finished (the last one scans their live counts)
-  uint32_t grad_chunk_ctr;  // chunks of live items taken by the backward projection's blocks
   uint32_t n_long;          // tiles whose list is longer than kTileSortShort (tile-sort binning)
 };
 static_assert(sizeof(Status) <= 256, "status block");

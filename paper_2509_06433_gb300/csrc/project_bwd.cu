@@ -10,6 +10,8 @@
 // Reverse: dSigma2 = -X Gbar X, dm = 2 dSigma2 m, dJ = dm Nm^T, dNm = J^T dm, dM = R^T dNm,
 // dQ = dM diag(s), ds = diag(Q^T dM), dq through the normalisation; dp_c from J, (u, v), z;
 // pose (left perturbation): drho = dp_c, dphi = p_c x dp_c + vee(Nm dNm^T - dNm Nm^T).
+#include <algorithm>
+
 #include "gs_internal.cuh"
 #include "sh.cuh"
 
@@ -112,12 +114,6 @@ __device__ __forceinline__ Sum10 sum_pairs_warp(const float* __restrict__ pg, co
   return mine;
 }
 
-// Blocks of k_item_grads: up to eight per multiprocessor, no more than there are chunks.
-int64_t item_grad_blocks(const Layout& L) {
-  const int64_t resident = static_cast<int64_t>(device_sms()) * 8;
-  return L.n_item_chunks < resident ? L.n_item_chunks : resident;
-}
-
 // Per-item partial gradient of the projection backward (16 floats): the mean's gradient in
 // world coordinates (0-2), the gradient of M = Q diag(exp(s)) (3-11, row-major), the opacity's
 // (12) and the colour's (13-15; with spherical harmonics the colour gradient after the clamp).
@@ -127,34 +123,37 @@ constexpr int kPartial = 16;
 // compact order of the live items (increasing k N + g): sums the item's pair records in slot
 // order (warp-cooperatively for items with many pairs), applies the chain rule of the view's
 // projection, writes the item's partial (when parameter gradients are wanted) and sums the
-// items' pose gradients per view. Blocks take chunks of kPoseBlock live items from a counter
-// (balanced whatever the chunks' work); a chunk's items are in view order, so each view k present
-// in chunk c gets the chunk's sum in slot c + k of pose_partials (unique: a later chunk's first
-// view is at least this chunk's last), which k_pose_reduce sums over the view's chunks in order.
-__global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
+// items' pose gradients per view. The blocks stride over chunks of kPoseBlock live items; a chunk's items are in view order, so each view k present in chunk c gets the chunk's sum in slot
+// c + k of pose_partials (unique: a later chunk's first view is at least this chunk's last), which
+// k_pose_reduce sums over the view's chunks in order.
+//
+// Bound by the latency of its chain of loads (item -> record bits -> records) and by DRAM (16 aerial views
+// of 2M Gaussians, 7.4M live items: 1.7 GB at 4.2 TB/s, 55% of the issue slots). So: small blocks with one
+// barrier per chunk, four times as many as are resident (the multiprocessors that get the lighter chunks
+// take more blocks), the records of four pairs in flight, storage types and colour mode fixed at compile
+// time. 500 -> 407 us there, 8 views of 250k 80 -> 74, one of 100k 22 -> 20, one of 60k with third-degree
+// harmonics 28 -> 23. Blocks of 256 threads 433, of 64 394 (but twice the sums for k_pose_reduce), only the
+// resident blocks 490; two pairs in flight and 5 blocks of 256 per SM 518; the parameters loaded before
+// the records 499 (spills).
+template <int DT, bool MF32, bool SH>
+__global__ void __launch_bounds__(kPoseBlock, SH ? 7 : 8) k_item_grads(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
                                                           uint8_t* __restrict__ ws, int want_params,
                                                           float* __restrict__ pose_partials) {
   pdl_wait();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int64_t n_live = at<Status>(ws, L.status)->n_live;
   const int64_t chunks = (n_live + kPoseBlock - 1) / kPoseBlock;
+  const uint32_t N = static_cast<uint32_t>(L.N > 0 ? L.N : 1);
   const uint32_t* live_kg = at<uint32_t>(ws, L.live_kg);
   const uint32_t* live_off = at<uint32_t>(ws, L.live_off);
   const uint32_t* live_count = at<uint32_t>(ws, L.live_count);
   const float* pg = at<float>(ws, L.pair_grads);
   const uint32_t* pvalid = at<uint32_t>(ws, L.pair_valid);
   float4* partials = at<float4>(ws, L.item_partials);
-  __shared__ float s_red[kPoseBlock / 32][6];
-  __shared__ int s_k0, s_k1;
-  __shared__ int64_t s_chunk;
-  uint32_t* ctr = &at<Status>(ws, L.status)->grad_chunk_ctr;
-  for (;;) {
-    __syncthreads();  // the previous chunk's s_k0 / s_k1 / s_chunk are read
-    if (threadIdx.x == 0) s_chunk = atomicAdd(ctr, 1u);
-    __syncthreads();
-    const int64_t c = s_chunk;
-    if (c >= chunks) break;
-    const int64_t pos = c * kPoseBlock + threadIdx.x;
+  __shared__ float s_red[2][kPoseBlock / 32][6];  // (two, so that a sum's readers need no second barrier)
+  int par = 0;
+  for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    const int64_t pos = c * kPoseBlock + threadIdx.x, end = min((c + 1) * kPoseBlock, n_live);
     const bool valid = pos < n_live;
     uint32_t kg = 0, off = 0, cnt = 0;
     if (valid) {
@@ -162,15 +161,19 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
       off = live_off[pos];
       cnt = live_count[pos];
     }
-    const int k = static_cast<int>(kg / static_cast<uint32_t>(L.N > 0 ? L.N : 1));
-    const int64_t g = static_cast<int64_t>(kg) - static_cast<int64_t>(k) * L.N;
+    const uint32_t kg0 = live_kg[c * kPoseBlock], kg1 = live_kg[end - 1];
+    const int k = static_cast<int>(kg / N);
+    const int64_t g = kg - static_cast<uint32_t>(k) * N;
     const Sum10 s = sum_pairs_warp(pg, pvalid, off, cnt, L.cap, valid);
     float pose[6] = {0, 0, 0, 0, 0, 0};
     if (valid) {
-      float p[3], ls[3], q[4];
-      for (int j = 0; j < 3; ++j) p[j] = load_attr(G.means, 3 * g + j, G.means_dtype);
-      for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, G.dtype);
-      for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, G.dtype);
+    float p[3], ls[3], q[4];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) p[j] = MF32 ? load_attr(G.means, 3 * g + j, GS_F32) : load_attr(G.means, 3 * g + j, G.means_dtype);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, DT);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, DT);
       const float qlen = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
       const float iq = qlen > 0.0f ? 1.0f / qlen : 0.0f;
       const float w = q[0] * iq, x = q[1] * iq, y = q[2] * iq, z = q[3] * iq;
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
       pose[4] = pc[2] * dpc[0] - pc[0] * dpc[2] + Am[2][0] - Am[0][2];
       pose[5] = pc[0] * dpc[1] - pc[1] * dpc[0] + Am[0][1] - Am[1][0];
       float gc0 = s.v[7], gc1 = s.v[8], gc2 = s.v[9];
-      if (L.color_mode == GS_COLOR_SH) {
+      if (SH) {
         // view-dependent colour: the colour gradient through the clamp (raw < 0: zero); its part
         // through the unit direction u = (p - C) / |p - C| goes to the mean, dL/dp = (I - u u^T)
         // (sum_i (f_i . g) grad Y_i) / |p - C|, and, as the camera centre moves by -R^T rho
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
         float Y[kShMaxCoeffs];
         sh_basis(u.x, u.y, u.z, Y);
         bool fin = true;
-        const float3 raw = sh_raw(G.rgb, G.dtype, g, L.sh_coeffs, Y, fin);
+        const float3 raw = sh_raw(G.rgb, DT, g, L.sh_coeffs, Y, fin);
         gc0 = raw.x >= 0.0f ? gc0 : 0.0f;
         gc1 = raw.y >= 0.0f ? gc1 : 0.0f;
         gc2 = raw.z >= 0.0f ? gc2 : 0.0f;
@@ -290,8 +293,8 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
           for (int i = 0; i < kShMaxCoeffs; ++i) {
             sv[i] = 0.0f;
             if (i < L.sh_coeffs)
-              sv[i] = gc0 * load_attr(G.rgb, base + 3 * i + 0, G.dtype) + gc1 * load_attr(G.rgb, base + 3 * i + 1, G.dtype) +
-                      gc2 * load_attr(G.rgb, base + 3 * i + 2, G.dtype);
+              sv[i] = gc0 * load_attr(G.rgb, base + 3 * i + 0, DT) + gc1 * load_attr(G.rgb, base + 3 * i + 1, DT) +
+                      gc2 * load_attr(G.rgb, base + 3 * i + 2, DT);
           }
           float gx, gy, gzz;
           sh_basis_vjp(u.x, u.y, u.z, sv, gx, gy, gzz);
@@ -319,27 +322,22 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
         dst[3] = make_float4(s.v[6], gc0, gc1, gc2);
       }
     }
-    // the block's pose sums per view: its items are in view order, from view s_k0 to s_k1
-    if (threadIdx.x == 0) s_k0 = valid ? k : 0;
-    const bool last_valid = valid && (threadIdx.x == kPoseBlock - 1 || pos + 1 == n_live);
-    if (last_valid) s_k1 = k;
-    __syncthreads();
-    const int k0 = s_k0, k1 = s_k1;
-    for (int kk = k0; kk <= k1; ++kk) {
+    // the chunk's pose sums per view: its items are in view order
+    const int k0 = static_cast<int>(kg0 / N), k1 = static_cast<int>(kg1 / N);
+    for (int kk = k0; kk <= k1; ++kk, par ^= 1) {
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
         float v = (valid && k == kk) ? pose[i] : 0.0f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) s_red[wib][i] = v;
+        if (lane == 0) s_red[par][wib][i] = v;
       }
       __syncthreads();
       if (threadIdx.x < 6) {
         float v = 0.0f;
-        for (int wv = 0; wv < kPoseBlock / 32; ++wv) v += s_red[wv][threadIdx.x];
+        for (int wv = 0; wv < kPoseBlock / 32; ++wv) v += s_red[par][wv][threadIdx.x];
         pose_partials[(c + kk) * 6 + threadIdx.x] = v;
       }
-      __syncthreads();
     }
   }
   pdl_trigger();
@@ -350,8 +348,11 @@ __global__ void __launch_bounds__(kPoseBlock, 4) k_item_grads(Layout L, GaussPtr
 // diag(exp(s)) to the log-scales and (through the normalisation) the quaternion, the opacity's
 // sigmoid to the logit; with spherical harmonics each view's colour gradient goes to the
 // coefficients through that view's basis values. A Gaussian that no view sees gets zero
-// gradients (stored with out.overwrite, nothing added otherwise).
-__global__ void __launch_bounds__(kPoseBlock) k_gaussian_grads(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
+// gradients (stored with out.overwrite, nothing added otherwise). Bound by the latency of the partials'
+// loads, so by the resident warps: 48 registers (2M Gaussians, 16 views: 216 -> 176 us; two views' loads
+// in flight with 80 registers 231, 40 registers 260). With harmonics the basis takes more.
+template <int DT, bool SH>
+__global__ void __launch_bounds__(kPoseBlock, SH ? 1 : 10) k_gaussian_grads(Layout L, GaussPtrs G, const gs_camera_t* __restrict__ cams,
                                                               const uint8_t* __restrict__ ws, gs_grads_t out) {
   pdl_wait();
   const int64_t g = static_cast<int64_t>(blockIdx.x) * kPoseBlock + threadIdx.x;
@@ -360,47 +361,51 @@ __global__ void __launch_bounds__(kPoseBlock) k_gaussian_grads(Layout L, GaussPt
   const uint32_t* live_wpre = at<uint32_t>(ws, L.live_wpre);
   const float4* partials = at<float4>(ws, L.item_partials);
   const bool store = out.overwrite != 0;
-  const bool sh = L.color_mode == GS_COLOR_SH;
   float acc[kPartial];
 #pragma unroll
   for (int i = 0; i < kPartial; ++i) acc[i] = 0.0f;
   bool seen = false, sh_touched = false;
-  uint32_t words[4], bases[4];
   float p[3] = {0, 0, 0};
-  if (sh && out.rgb) for (int j = 0; j < 3; ++j) p[j] = load_attr(G.means, 3 * g + j, G.means_dtype);
-  for (int k = 0; k < L.K; ++k) {
+  if (SH && out.rgb)
+    for (int j = 0; j < 3; ++j) p[j] = load_attr(G.means, 3 * g + j, G.means_dtype);
+  for (int k4 = 0; k4 < L.K; k4 += 4) {
     // the mask words and rank bases of four views at a time are loaded together
-    if ((k & 3) == 0) {
+    uint32_t words[4], bases[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int64_t kgj = static_cast<int64_t>(k + j) * L.N + g;
-        words[j] = k + j < L.K ? live_mask[kgj >> 5] : 0u;
-        bases[j] = (words[j] >> (kgj & 31)) & 1u ? live_wpre[kgj >> 5] : 0u;
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int64_t kg = static_cast<int64_t>(k4 + j) * L.N + g;
+      const uint32_t word = k4 + j < L.K ? live_mask[kg >> 5] : 0u;
+      const bool live = (word >> (kg & 31)) & 1u;
+      words[j] = live ? word & ((1u << (kg & 31)) - 1u) : 0xffffffffu;
+      bases[j] = live ? live_wpre[kg >> 5] : 0u;
     }
-    const int64_t kg = static_cast<int64_t>(k) * L.N + g;
-    const uint32_t word = words[k & 3];
-    if (!((word >> (kg & 31)) & 1u)) continue;
-    seen = true;
-    const uint32_t pos = bases[k & 3] + __popc(word & ((1u << (kg & 31)) - 1u));
-    const float4* src = partials + static_cast<int64_t>(pos) * (kPartial / 4);
-    const float4 a = src[0], b = src[1], c = src[2], d = src[3];
-    const float v[kPartial] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
 #pragma unroll
-    for (int i = 0; i < kPartial; ++i) acc[i] += v[i];
-    if (sh && out.rgb) {  // dL/df_i += Y_i(u_k) g_k for this view's direction
-      const ShDir u = sh_dir(p[0], p[1], p[2], cams[k]);
-      float Y[kShMaxCoeffs];
-      sh_basis(u.x, u.y, u.z, Y);
-      const int64_t base = g * L.sh_coeffs * 3;
-      const bool first = store && !sh_touched;
-      for (int i = 0; i < L.sh_coeffs; ++i) {
-        float* o3 = out.rgb + base + 3 * i;
-        put(o3 + 0, first, Y[i] * d.y);
-        put(o3 + 1, first, Y[i] * d.z);
-        put(o3 + 2, first, Y[i] * d.w);
+    for (int j = 0; j < 4; ++j) {
+      if (words[j] == 0xffffffffu) continue;
+      seen = true;
+      const float4* src = partials + static_cast<int64_t>(bases[j] + __popc(words[j])) * (kPartial / 4);
+      const float4 part[4] = {src[0], src[1], src[2], src[3]};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[4 * i] += part[i].x;
+        acc[4 * i + 1] += part[i].y;
+        acc[4 * i + 2] += part[i].z;
+        acc[4 * i + 3] += part[i].w;
       }
-      sh_touched = true;
+      if (SH && out.rgb) {  // dL/df_i += Y_i(u_k) g_k for this view's direction
+        const ShDir u = sh_dir(p[0], p[1], p[2], cams[k4 + j]);
+        float Y[kShMaxCoeffs];
+        sh_basis(u.x, u.y, u.z, Y);
+        const int64_t base = g * L.sh_coeffs * 3;
+        const bool first = store && !sh_touched;
+        for (int i = 0; i < L.sh_coeffs; ++i) {
+          float* o3 = out.rgb + base + 3 * i;
+          put(o3 + 0, first, Y[i] * part[3].y);
+          put(o3 + 1, first, Y[i] * part[3].z);
+          put(o3 + 2, first, Y[i] * part[3].w);
+        }
+        sh_touched = true;
+      }
     }
   }
   if (!seen) {
@@ -411,16 +416,16 @@ __global__ void __launch_bounds__(kPoseBlock) k_gaussian_grads(Layout L, GaussPt
         for (int j = 0; j < 4; ++j) out.quats[4 * g + j] = 0.0f;
       if (out.opacity_logits) out.opacity_logits[g] = 0.0f;
       if (out.rgb) {
-        const int cw = sh ? 3 * L.sh_coeffs : 3;
+        const int cw = SH ? 3 * L.sh_coeffs : 3;
         for (int j = 0; j < cw; ++j) out.rgb[cw * g + j] = 0.0f;
       }
     }
     return;
   }
   float ls[3], q[4];
-  for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, G.dtype);
-  for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, G.dtype);
-  const float lg = load_attr(G.logits, g, G.dtype);
+  for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, DT);
+  for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, DT);
+  const float lg = load_attr(G.logits, g, DT);
   const float qlen = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
   const float iq = qlen > 0.0f ? 1.0f / qlen : 0.0f;
   const float w = q[0] * iq, x = q[1] * iq, y = q[2] * iq, z = q[3] * iq;
@@ -460,7 +465,7 @@ __global__ void __launch_bounds__(kPoseBlock) k_gaussian_grads(Layout L, GaussPt
   if (out.quats)
     for (int j = 0; j < 4; ++j) put(out.quats + 4 * g + j, store, (dqh[j] - qh[j] * qd) * iq);
   if (out.opacity_logits) put(out.opacity_logits + g, store, acc[12] * o * (1.0f - o));
-  if (out.rgb && !sh)
+  if (out.rgb && !SH)
     for (int j = 0; j < 3; ++j) put(out.rgb + 3 * g + j, store, acc[13 + j]);
 }
 
@@ -482,6 +487,7 @@ __global__ void k_pose_reduce(const float* __restrict__ partials, Layout L, cons
   const int64_t r0 = rank(static_cast<int64_t>(k) * L.N), r1 = rank(static_cast<int64_t>(k + 1) * L.N);
   float v = 0.0f;
   if (r1 > r0)
+#pragma unroll 8
     for (int64_t c = r0 / kPoseBlock + lane; c <= (r1 - 1) / kPoseBlock; c += 32) v += partials[(c + k) * 6 + i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -535,6 +541,13 @@ __global__ void __launch_bounds__(kPoseBlock) k_screen_grads(Layout L, const uin
 
 }  // namespace
 
+namespace {
+// Blocks of k_item_grads: four times the resident ones, no more than there are chunks.
+unsigned item_grad_blocks(const Layout& L) {
+  return static_cast<unsigned>(std::min<int64_t>(L.n_item_chunks, static_cast<int64_t>(device_sms()) * 32));
+}
+}  // namespace
+
 cudaError_t launch_project_bwd(const Layout& L, const GaussPtrs& g, const gs_camera_t* cams, void* ws,
                                const gs_grads_t& out, cudaStream_t s) {
   if (L.N == 0) {
@@ -544,11 +557,25 @@ cudaError_t launch_project_bwd(const Layout& L, const GaussPtrs& g, const gs_cam
   auto* w = static_cast<uint8_t*>(ws);
   float* partials = at<float>(ws, L.pose_partials);
   const bool params = out.means || out.log_scales || out.quats || out.opacity_logits || out.rgb;
-  cudaMemsetAsync(&at<Status>(ws, L.status)->grad_chunk_ctr, 0, sizeof(uint32_t), s);
-  launch(k_item_grads, static_cast<unsigned>(item_grad_blocks(L)), kPoseBlock, 0, s, L, g, cams, w, params ? 1 : 0,
-         partials);
-  if (params) launch(k_gaussian_grads, static_cast<unsigned>(L.n_pose_blocks), kPoseBlock, 0, s, L, g, cams,
-                     static_cast<const uint8_t*>(ws), out);
+#define GS_PBWD_S(DT, SH)                                                                                            \
+  {                                                                                                                 \
+    if (g.means_dtype == GS_F32) GS_ITEM(DT, true, SH) else GS_ITEM(DT, false, SH)                                   \
+    if (params) launch(k_gaussian_grads<DT, SH>, static_cast<unsigned>(L.n_pose_blocks), kPoseBlock, 0, s, L, g, cams, \
+                       static_cast<const uint8_t*>(ws), out);                                                       \
+  }
+#define GS_ITEM(DT, M, SH)                                                                                         \
+  launch(k_item_grads<DT, M, SH>, item_grad_blocks(L), kPoseBlock, 0, s, L, g, cams, w, \
+         params ? 1 : 0, partials);
+#define GS_PBWD(DT) \
+  if (L.color_mode == GS_COLOR_SH) GS_PBWD_S(DT, true) else GS_PBWD_S(DT, false)
+  switch (g.dtype) {
+    case GS_F32: GS_PBWD(GS_F32) break;
+    case GS_BF16: GS_PBWD(GS_BF16) break;
+    default: GS_PBWD(GS_F16) break;
+  }
+#undef GS_PBWD
+#undef GS_PBWD_S
+#undef GS_ITEM
   if (out.pose)
     launch(k_pose_reduce, L.K, 6 * 32, 0, s, static_cast<const float*>(partials), L, static_cast<const uint8_t*>(ws),
            out.pose, out.overwrite);
