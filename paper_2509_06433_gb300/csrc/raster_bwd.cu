@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(kTilePixels / PX, PX == 4 ? kMinBlocksPx4 : (P
                                                                  const float* __restrict__ g_depth,
                                                                  const float* __restrict__ g_T) {
   pdl_wait();
-  __shared__ BwdSmem<PX, CH> M;
+  __shared__ BwdSmem<PX, CH, false> M;
   const TileCoord tc = tile_coord(L, blockIdx.x);
   const int lx = threadIdx.x & (kTile - 1), ly = (threadIdx.x / kTile) * PX;
   const int px = tc.tx * kTile + lx, py = tc.ty * kTile + ly;
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kTilePixels / PX, PX == 4 ? kMinBlocksPx4 : (P
       last[q] = last_in[tc.k * HW + pix];
     }
   }
-  bwd_sweep<PX, CH>(M, L, ws, tc, rg, Sg, hT, gr, gg, gb, gd, last);
+  bwd_sweep<PX, CH, true, false>(M, L, ws, tc, rg, Sg, hT, gr, gg, gb, gd, last);
   pdl_trigger();
 }
 

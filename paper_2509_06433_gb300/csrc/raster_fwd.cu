@@ -50,17 +50,17 @@ using RasterWs = typename std::conditional<(CHB > 0), uint8_t*, const uint8_t*>:
 // Shared memory of the forward: its staged chunk; with the fused backward, the backward sweep's
 // shared memory in the same bytes (the forward's chunks are dead once every thread has passed
 // the loss reduction's barriers, before the sweep starts).
-template <int PX, int CH, int CHB>
+template <int PX, int CH, int CHB, bool ROWS>
 union FusedSmem {
   Stage<CH> S;
-  BwdSmem<PX, CHB> M;
+  BwdSmem<PX, CHB, ROWS> M;
 };
-template <int PX, int CH, int CHB>
+template <int PX, int CH, int CHB, bool ROWS>
 struct FwdSmemOf {
-  using T = FusedSmem<PX, CH, CHB>;
+  using T = FusedSmem<PX, CH, CHB, ROWS>;
 };
-template <int PX, int CH>
-struct FwdSmemOf<PX, CH, 0> {
+template <int PX, int CH, bool ROWS>
+struct FwdSmemOf<PX, CH, 0, ROWS> {
   struct T {
     Stage<CH> S;
   };
@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   constexpr int kThreads = kTilePixels / PX;
   constexpr int kWarps = kThreads / 32;
   const float kInf = __int_as_float(0x7f800000);
-  __shared__ typename FwdSmemOf<PX, CH, CHB>::T sm;
+  constexpr bool kRows = PX == 2 || (PX == 4 && !MANY);  // (see warp_reduce10_rows)
+  __shared__ typename FwdSmemOf<PX, CH, CHB, kRows>::T sm;
   Stage<CH>& S = sm.S;
   __shared__ uint32_t s_red[2][kWarps];
   const TileCoord tc = tile_coord(L, blockIdx.x);
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   if constexpr (CHB > 0) {
     // the backward pass of this tile, from registers: the weighted colour behind the first
     // splat is the loss gradient applied to the pixel's output (no dL/dT_final term)
-    BwdSmem<PX, CHB>& M = sm.M;
+    BwdSmem<PX, CHB, kRows>& M = sm.M;
     float Sg[PX], hT[PX], gr[PX], gg[PX], gb[PX], gd[PX];
     int lst[PX];
 #pragma unroll
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(kTilePixels / PX,
       hT[q] = 0.0f;
       lst[q] = in ? last[q] : 0;
     }
-    bwd_sweep<PX, CHB, false>(M, L, ws, tc, rg, Sg, hT, gr, gg, gb, gd, lst);
+    bwd_sweep<PX, CHB, false, kRows>(M, L, ws, tc, rg, Sg, hT, gr, gg, gb, gd, lst);
     pdl_trigger();
   }
   if (STATS) {

@@ -52,14 +52,45 @@ __device__ __forceinline__ int reduce10_index(int lane) {
 }
 __device__ __forceinline__ bool reduce10_writer(int lane) { return !(lane & 1) && (!(lane & 2) || !(lane & 12)); }
 
+// The same sums, bit for bit, through shared memory: every lane stores its 10 values as a row of buf, then
+// lane 8 r + c (r < 4, c < 5) adds value pair c over the rows l with l % 4 = r, in the tree that the shuffles
+// take (lane bits 4, 3, 2), and two shuffles add the groups (bits 1, 0). 27 instructions instead of 43, but
+// three times the shared-memory cycles. A row is 64 bytes and a group of 8 rows 560, so that neither the
+// stores (16 bytes per lane) nor the loads (8 bytes) meet in a bank. On return lane 8 r + c, c < 5, r % 2 = 0,
+// holds value 2 c + r / 2.
+//
+// Where: the loss-fused kernel at 2 pixels per thread, and at 4 without the blocks-per-SM register budget;
+// few warps per SM there wait for their own instructions (1200 tiles, us: 147.4 -> 143.3 and 120.8 -> 116.8 at
+// 4 pixels, 159.9 -> 153.7 at 2; 9600 tiles at 2 741 -> 722). With the budget the saved instructions are lost
+// to shared memory (16 aerial views 3.83 -> 3.97 ms), and so they are in the backward alone (9600 tiles at 2
+// pixels 485 -> 509).
+constexpr int kRowFloats = 16, kRowGroupFloats = 8 * kRowFloats + 12;
+__device__ __forceinline__ float warp_reduce10_rows(const float (&x)[10], int lane, float* buf) {
+  float* row = buf + (lane & 3) * kRowGroupFloats + (lane >> 2) * kRowFloats;
+  __syncwarp();  // the last call's loads are done
+  reinterpret_cast<float4*>(row)[0] = make_float4(x[0], x[1], x[2], x[3]);
+  reinterpret_cast<float4*>(row)[1] = make_float4(x[4], x[5], x[6], x[7]);
+  reinterpret_cast<float2*>(row)[4] = make_float2(x[8], x[9]);
+  __syncwarp();
+  const float* col = buf + (lane >> 3) * kRowGroupFloats + 2 * min(lane & 7, 4);
+  float2 v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = *reinterpret_cast<const float2*>(col + i * kRowFloats);
+  const float2 s = vadd(vadd(vadd(v[0], v[4]), vadd(v[2], v[6])), vadd(vadd(v[1], v[5]), vadd(v[3], v[7])));
+  const bool high = lane & 16;
+  const float u = (high ? s.y : s.x) + __shfl_xor_sync(0xffffffffu, high ? s.x : s.y, 16);
+  return u + __shfl_xor_sync(0xffffffffu, u, 8);
+}
+
 // Shared memory of one backward sweep: the staged chunk, the chunk's record slots, the warp
 // partials of its 10 sums and the warps' largest `last`.
-template <int PX, int CH>
+template <int PX, int CH, bool ROWS>
 struct BwdSmem {
   static constexpr int kWarps = kTilePixels / PX / 32;
   Stage<CH> S;
   uint32_t slot[CH];
   float part[kWarps][CH][10];
+  __align__(16) float rows[ROWS ? kWarps : 1][ROWS ? 4 * kRowGroupFloats : 4];
   uint32_t written[kWarps][CH / 32];  // splats of the chunk whose part a warp has written
   int maxlast[kWarps];
 };
@@ -89,8 +120,9 @@ __device__ __forceinline__ float weighted_colour(float gr, float gg, float gb, f
 // one record per pair in front of some pixel's last contributor. All threads of the block call it.
 // HT = false: every hT is zero (no dL/dT_final term) and the sweep leaves it out; the results are
 // the same bit for bit (a zero addend changes at most the sign of a zero, which the sums drop).
-template <int PX, int CH, bool HT = true>
-__device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, uint8_t* __restrict__ ws,
+// ROWS: the warp sums go through shared memory (warp_reduce10_rows).
+template <int PX, int CH, bool HT, bool ROWS>
+__device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH, ROWS>& M, const Layout& L, uint8_t* __restrict__ ws,
                                           const TileCoord& tc, uint2 rg, const float (&Sg)[PX], const float (&hT)[PX],
                                           const float (&gr)[PX], const float (&gg)[PX], const float (&gb)[PX],
                                           const float (&gd)[PX], const int (&last)[PX]) {
@@ -134,8 +166,8 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) max_last = max(max_last, M.maxlast[w]);
   const uint32_t stop = min(rg.y, rg.x + static_cast<uint32_t>(max_last));
-  const int idx = reduce10_index(lane);
-  const bool writer = reduce10_writer(lane);
+  const int idx = ROWS ? 2 * (lane & 7) + (lane >> 4) : reduce10_index(lane);
+  const bool writer = ROWS ? (lane & 7) < 5 && !(lane & 8) : reduce10_writer(lane);
   constexpr float kLn2 = 0.6931471805599453f;
 
   // One splat of the staged chunk at list position pos; returns whether a pixel of the warp keeps it.
@@ -207,7 +239,9 @@ __device__ __forceinline__ void bwd_sweep(BwdSmem<PX, CH>& M, const Layout& L, u
     const float dx = comp(col.dx, 0);
     const float dxP0 = dx * p0;
     const float v[10] = {dxP0, p1, dx * dxP0, dx * p1, hsum(P2), hsum(ncz), p0, hsum(ncr), hsum(ncg), hsum(ncb)};
-    const float r = warp_reduce10(v, lane);
+    float r;
+    if constexpr (ROWS) r = warp_reduce10_rows(v, lane, M.rows[warp]);
+    else r = warp_reduce10(v, lane);
     if (writer) M.part[warp][j][idx] = r;
     return true;
   };
