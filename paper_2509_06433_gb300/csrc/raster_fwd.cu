@@ -66,6 +66,57 @@ struct FwdSmemOf<PX, CH, 0, ROWS> {
   };
 };
 
+// A thread's pixels against one splat. Minus the alpha with which each keeps it (0 where it doesn't) and
+// whether it does; FULL evaluates the clamp and the power test too (see kChecked), OCC the occlusion.
+template <int PX>
+using Px = typename Vec<(PX >= 2 ? 2 : 1)>::T;
+template <int PX, bool FULL, bool OCC>
+__device__ __forceinline__ void pixel_alphas(const float4& A, const float4& B, Px<PX> npx,
+                                             const Px<PX> (&npy)[PX >= 2 ? PX / 2 : 1], const float (&zmax)[PX],
+                                             Px<PX> (&na)[PX >= 2 ? PX / 2 : 1], bool (&keep)[PX]) {
+  constexpr int W = PX >= 2 ? 2 : 1, G = PX / W;
+  const Column<W> col = splat_column<W>(A, B, npx);
+  const Px<PX> Ay = bcast<W>(A.y);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const Px<PX> e = splat_exponent<W>(B, col, vadd(Ay, npy[g]));
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const int q = g * W + i;
+      const float raw = ex2_approx(comp(e, i));
+      const float a = FULL ? fminf(raw, kAlphaMax) : raw;
+      keep[q] = a >= kAlphaMin;
+      if (FULL) keep[q] = keep[q] && comp(e, i) <= B.w;
+      if (OCC) keep[q] = keep[q] && !(B.z >= zmax[q]);  // a splat at or behind the surface
+      set_comp(na[g], i, keep[q] ? -a : 0.0f);
+    }
+  }
+}
+template <int PX>
+__device__ __forceinline__ bool any_below(const Px<PX> (&t)[PX >= 2 ? PX / 2 : 1]) {
+  constexpr int W = PX >= 2 ? 2 : 1;
+  float low = comp(t[0], 0);
+#pragma unroll
+  for (int q = 1; q < PX; ++q) low = fminf(low, comp(t[q / W], q % W));
+  return low < kTStop;
+}
+template <int PX>
+__device__ __forceinline__ void blend(const float4& C, const Px<PX> (&na)[PX >= 2 ? PX / 2 : 1],
+                                      const Px<PX> (&T)[PX >= 2 ? PX / 2 : 1], Px<PX> (&cr)[PX >= 2 ? PX / 2 : 1],
+                                      Px<PX> (&cg)[PX >= 2 ? PX / 2 : 1], Px<PX> (&cb)[PX >= 2 ? PX / 2 : 1],
+                                      Px<PX> (&cd)[PX >= 2 ? PX / 2 : 1]) {
+  constexpr int W = PX >= 2 ? 2 : 1, G = PX / W;
+  const Px<PX> nR = bcast<W>(C.x), nG = bcast<W>(C.y), nB = bcast<W>(C.z), nZ = bcast<W>(C.w);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const Px<PX> nw = vmul(na[g], T[g]);
+    cr[g] = vfma(nR, nw, cr[g]);
+    cg[g] = vfma(nG, nw, cg[g]);
+    cb[g] = vfma(nB, nw, cb[g]);
+    cd[g] = vfma(nZ, nw, cd[g]);
+  }
+}
+
 // MANY = false (the fused variant only): compiled without the blocks-per-SM register budget, for
 // grids that fit on the GPU in one wave anyway, where each block's own latency sets the time.
 template <int PX, int CH, bool STATS, bool LOSS, bool OCC = false, int CHB = 0, bool MANY = true>
@@ -79,6 +130,11 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   pdl_wait();
   constexpr int kThreads = kTilePixels / PX;
   constexpr int kWarps = kThreads / 32;
+  // Two splats per turn (splat2): a warp waits less for its own chain of loads, exponentials and votes, and the
+  // vote and the loop are paid once for two. Forward at 2 / 4 pixels, us: 300 tiles 28.6 -> 26.5 / 36.8 -> 30.7,
+  // 3600 uneven 111 -> 107 / 126 -> 114, 9600 235 -> 225 / 201 -> 187, 57600 1547 -> 1475 / 1343 -> 1270; fused at 2
+  // pixels 2 to 6%. Not in the fused kernel under the blocks-per-SM register budget (spills: 3.84 -> 3.88 ms).
+  constexpr bool kPairs = !OCC && !STATS && PX >= 2 && !(CHB > 0 && PX == 4 && MANY);
   const float kInf = __int_as_float(0x7f800000);
   constexpr bool kRows = PX == 2 || (PX == 4 && !MANY);  // (see warp_reduce10_rows)
   __shared__ typename FwdSmemOf<PX, CH, CHB, kRows>::T sm;
@@ -141,36 +197,15 @@ __global__ void __launch_bounds__(kTilePixels / PX,
   // (-c)(na T) are the same roundings as with positive operands, without a negated copy of T.
   const int lane = threadIdx.x & 31;
   auto splat = [&](auto full, int j, int pos) {
-    constexpr bool FULL = decltype(full)::value;
     const float4 A = S.A[j], B = S.B[j], C = S.C[j];
-    const Column<W> col = splat_column<W>(A, B, npx);
-    const V Ay = bcast<W>(A.y);
     V na[G], Tn[G];
     bool keep[PX];
+    pixel_alphas<PX, decltype(full)::value, OCC>(A, B, npx, npy, zmax, na, keep);
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const V e = splat_exponent<W>(B, col, vadd(Ay, npy[g]));
-#pragma unroll
-      for (int i = 0; i < W; ++i) {
-        const int q = g * W + i;
-        const float raw = ex2_approx(comp(e, i));
-        const float a = FULL ? fminf(raw, kAlphaMax) : raw;
-        keep[q] = a >= kAlphaMin;
-        if (FULL) keep[q] = keep[q] && comp(e, i) <= B.w;
-        if (OCC) keep[q] = keep[q] && !(B.z >= zmax[q]);  // a splat at or behind the surface
-        set_comp(na[g], i, keep[q] ? -a : 0.0f);
-      }
-      Tn[g] = vfma(T[g], na[g], T[g]);
-    }
+    for (int g = 0; g < G; ++g) Tn[g] = vfma(T[g], na[g], T[g]);
     // a pixel stops before the splat that would leave T < 1e-4 (once per pixel, so the changes are
     // made in a warp-uniform branch; a skipped splat leaves T, which is never below 1e-4)
-    bool event = false;
-    {
-      float low = comp(Tn[0], 0);
-#pragma unroll
-      for (int q = 1; q < PX; ++q) low = fminf(low, comp(Tn[q / W], q % W));
-      event = low < kTStop;
-    }
+    bool event = any_below<PX>(Tn);
     if (OCC) {
 #pragma unroll
       for (int q = 0; q < PX; ++q) event = event || (B.z >= zmax[q] && comp(npy[q / W], q % W) != kInf);
@@ -187,20 +222,68 @@ __global__ void __launch_bounds__(kTilePixels / PX,
 #pragma unroll
       for (int g = 0; g < G; ++g) Tn[g] = vfma(T[g], na[g], T[g]);
     }
-    const V nR = bcast<W>(C.x), nG = bcast<W>(C.y), nB = bcast<W>(C.z), nZ = bcast<W>(C.w);
+    blend<PX>(C, na, T, cr, cg, cb, cd);
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const V nw = vmul(na[g], T[g]);
-      cr[g] = vfma(nR, nw, cr[g]);
-      cg[g] = vfma(nG, nw, cg[g]);
-      cb[g] = vfma(nB, nw, cb[g]);
-      cd[g] = vfma(nZ, nw, cd[g]);
-      T[g] = Tn[g];
-    }
+    for (int g = 0; g < G; ++g) T[g] = Tn[g];
 #pragma unroll
     for (int q = 0; q < PX; ++q) {
       last[q] = keep[q] ? pos + 1 : last[q];
       if (STATS) blended += keep[q] ? 1u : 0u;
+    }
+  };
+  auto all_stopped = [&]() -> bool {
+    all_done = true;
+#pragma unroll
+    for (int q = 0; q < PX; ++q) all_done = all_done && comp(npy[q / W], q % W) == kInf;
+    return __all_sync(0xffffffffu, all_done);
+  };
+  // Two successive splats of the warp's list (j0 before j1), bit for bit as one after the other: their
+  // opacities don't depend on each other, so that the two chains of loads, exponentials and tests overlap, and
+  // one vote serves both (T only falls, so a pixel that stops at either has the second T below 1e-4).
+  auto splat2 = [&](auto full, int j0, int j1, int pos) {
+    const float4 A0 = S.A[j0], B0 = S.B[j0], A1 = S.A[j1], B1 = S.B[j1];
+    V n0[G], n1[G], T1[G], T2[G];
+    bool keep0[PX], keep1[PX];
+    pixel_alphas<PX, decltype(full)::value, OCC>(A0, B0, npx, npy, zmax, n0, keep0);
+    pixel_alphas<PX, decltype(full)::value, OCC>(A1, B1, npx, npy, zmax, n1, keep1);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      T1[g] = vfma(T[g], n0[g], T[g]);
+      T2[g] = vfma(T1[g], n1[g], T1[g]);
+    }
+    if (__any_sync(0xffffffffu, any_below<PX>(T2))) {
+#pragma unroll
+      for (int q = 0; q < PX; ++q) {
+        const bool stop = comp(T1[q / W], q % W) < kTStop;
+        keep0[q] = keep0[q] && !stop;
+        keep1[q] = keep1[q] && !stop;
+        set_comp(n0[q / W], q % W, stop ? 0.0f : comp(n0[q / W], q % W));
+        set_comp(n1[q / W], q % W, stop ? 0.0f : comp(n1[q / W], q % W));
+        set_comp(npy[q / W], q % W, stop ? kInf : comp(npy[q / W], q % W));
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        T1[g] = vfma(T[g], n0[g], T[g]);
+        T2[g] = vfma(T1[g], n1[g], T1[g]);
+      }
+#pragma unroll
+      for (int q = 0; q < PX; ++q) {
+        const bool stop = comp(T2[q / W], q % W) < kTStop;
+        keep1[q] = keep1[q] && !stop;
+        set_comp(n1[q / W], q % W, stop ? 0.0f : comp(n1[q / W], q % W));
+        set_comp(npy[q / W], q % W, stop ? kInf : comp(npy[q / W], q % W));
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) T2[g] = vfma(T1[g], n1[g], T1[g]);
+    }
+    blend<PX>(S.C[j0], n0, T, cr, cg, cb, cd);
+    blend<PX>(S.C[j1], n1, T1, cr, cg, cb, cd);
+#pragma unroll
+    for (int g = 0; g < G; ++g) T[g] = T2[g];
+#pragma unroll
+    for (int q = 0; q < PX; ++q) {
+      last[q] = keep0[q] ? pos + j0 + 1 : last[q];
+      last[q] = keep1[q] ? pos + j1 + 1 : last[q];
     }
   };
   for (uint32_t base = rg.x; base < rg.y; base += CH) {
@@ -213,30 +296,50 @@ __global__ void __launch_bounds__(kTilePixels / PX,
     const int n = min(CH, static_cast<int>(rg.y - base));
     const int pos0 = static_cast<int>(base - rg.x);
     // the splats that meet the warp's rows, 32 at a time (the loop runs over the set bits only; it
-    // ends early when every pixel of the warp has stopped, looked at after every 8 list positions)
+    // ends early when every pixel of the warp has stopped, looked at now and then)
     bool done = __all_sync(0xffffffffu, all_done);
 #pragma unroll 1
     for (int w0 = 0; w0 < n && !done; w0 += 32) {
       const uint32_t r = w0 + lane < n ? S.rows[w0 + lane] : 0u;
       uint32_t visit = __ballot_sync(0xffffffffu, (r & wrows) != 0);
       const uint32_t checked = __ballot_sync(0xffffffffu, (r & kChecked) != 0);
+      if constexpr (kPairs) {  // (a check every four turns, about every eight splats)
+        int j = __ffs(visit) - 1;
 #pragma unroll 1
-      for (int k = 0; visit && !done; k += 8) {
-        uint32_t v = visit & (0xffu << k);
-        visit &= ~(0xffu << k);
-        int j = __ffs(v) - 1;
-#pragma unroll 1
-        while (j >= 0) {
-          v &= v - 1;
-          const int next = __ffs(v) - 1;  // (found ahead of the splat's own chain)
-          if (OCC || ((checked >> j) & 1u)) splat(std::true_type{}, w0 + j, pos0 + w0 + j);
-          else splat(std::false_type{}, w0 + j, pos0 + w0 + j);
+        for (int turn = 1; j >= 0; ++turn) {
+          visit &= visit - 1;
+          int next = __ffs(visit) - 1;  // (found ahead of the splat's own chain)
+          if (next >= 0) {
+            visit &= visit - 1;
+            const int after = __ffs(visit) - 1;
+            if (((checked >> j) | (checked >> next)) & 1u) splat2(std::true_type{}, w0 + j, w0 + next, pos0);
+            else splat2(std::false_type{}, w0 + j, w0 + next, pos0);
+            next = after;
+          } else if ((checked >> j) & 1u) {
+            splat(std::true_type{}, w0 + j, pos0 + w0 + j);
+          } else {
+            splat(std::false_type{}, w0 + j, pos0 + w0 + j);
+          }
           j = next;
+          if ((turn & 3) == 0 && all_stopped()) break;
         }
-        all_done = true;
-#pragma unroll
-        for (int q = 0; q < PX; ++q) all_done = all_done && comp(npy[q / W], q % W) == kInf;
-        done = __all_sync(0xffffffffu, all_done);
+        done = all_stopped();
+      } else {  // (a check every eight list positions)
+#pragma unroll 1
+        for (int k = 0; visit && !done; k += 8) {
+          uint32_t v = visit & (0xffu << k);
+          visit &= ~(0xffu << k);
+          int j = __ffs(v) - 1;
+#pragma unroll 1
+          while (j >= 0) {
+            v &= v - 1;
+            const int next = __ffs(v) - 1;
+            if (OCC || ((checked >> j) & 1u)) splat(std::true_type{}, w0 + j, pos0 + w0 + j);
+            else splat(std::false_type{}, w0 + j, pos0 + w0 + j);
+            j = next;
+          }
+          done = all_stopped();
+        }
       }
     }
   }
