@@ -474,6 +474,8 @@ __host__ __device__ inline int64_t sort_tiles(int64_t n, int items) {
 // Keys per thread for a sort of up to n keys: small sorts take short tiles, so that enough
 // blocks share the work.
 // keys per thread: small sorts take small tiles (more blocks, shorter per-tile latency)
+// (from kSortLongTilesFrom pairs on, gs_sort_pairs also runs in scratch that only long tiles fit)
+constexpr int64_t kSortLongTilesFrom = 600000;
 inline int pick_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 1000000 ? 8 : kSortItems); }
 using SortArgs = SortArgsT<uint64_t>;
 using SortArgs32 = SortArgsT<uint32_t>;
