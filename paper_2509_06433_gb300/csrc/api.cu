@@ -74,7 +74,8 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
   // on (a list is sorted by one block) and while the lists stay short: projection + binning of 300k
   // Gaussians on planes at 640x480 (250 per tile, lists of 2018) takes 134 us against 198 by the
   // radix sorts, 600k 283 against 318, 1M (833 per tile, lists of 6723) 473 against 465, 2M 941
-  // against 850.
+  // against 850; Gaussians in free space (13 pairs each), 767 per tile (lists of 5142) 494 against 535,
+  // 1011 (lists of 12972) 1029 against 925.
   L->tile_sort = L->n_tiles >= kTileSortMinTiles && L->N > 0 && L->N <= kTileSortMaxItems &&
                  L->KN <= kTileSortMaxDensity * L->n_tiles;
   L->sort_groups = static_cast<int>((L->KN + kTileSortGroupItems - 1) / kTileSortGroupItems);

@@ -31,7 +31,7 @@ constexpr int kTileSortMinTiles = 152;  // fewer tiles than SMs: the global radi
 constexpr int kScanRows = 8;            // tile rows per block of the tile scan
 constexpr int kTileSubLists = 4;        // cursors per tile: projection block b emits into sub-list b % 4
 constexpr int kCursorStride = 8;        // u32 between two cursors: one 32-byte sector each
-constexpr int kTileSortMaxDensity = 1024;  // Gaussians per tile of a view (see make_layout)
+constexpr int kTileSortMaxDensity = 800;  // Gaussians per tile of a view (see make_layout)
 constexpr int64_t kTileSortMaxItems = 1 << 25;  // most Gaussians (so list entries; 27-bit bucket numbers)
 constexpr int kTileSortShort = 2048;    // longest list sorted by a short-list block
 constexpr int kTileSortGroupItems = 6400000;  // (view, Gaussian) items per emission / sort launch
