@@ -63,7 +63,7 @@ cudaError_t launch_raster_bwd(const Layout& L, void* ws, const float* rgb, const
     case 128: GS_BWD(P, 128); break; \
     default: GS_BWD(P, 64); break;   \
   }
-  switch (pick_px(L.bwd_px, default_px(L, true))) {
+  switch (pick_px(L.bwd_px, default_px(L))) {
     case 1: GS_BWD_CH(1); break;
     case 2: GS_BWD_CH(2); break;
     default: GS_BWD_CH(4); break;

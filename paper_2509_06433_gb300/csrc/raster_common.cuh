@@ -225,16 +225,16 @@ __device__ __forceinline__ TileCoord tile_coord(const Layout& L, int64_t tile_g)
   return c;
 }
 
-// Pixels per thread when the caller leaves the choice to the library: 4 unless the grid is small, where
-// 2 spreads a tile over twice the warps. With a backward sweep from 1024 tiles on (loss-fused forward +
-// backward, us at 2 / 4 pixels: 672 tiles 133 / 150, 1200 tiles 160 / 150 and 145 / 123, 4032 tiles 195 /
-// 168); forward only from 4000 (300 tiles 28.6 / 36.8, 1200 55 / 53, 3600 with uneven lists 112 / 127,
-// 4032 60 / 58, 9600 236 / 201).
+// Pixels per thread when the caller leaves the choice to the library: 4 only on large grids. It is the faster
+// one on most scenes from 3600 tiles on (loss-fused forward + backward, us at 2 / 4 pixels, 9 views of 640x480:
+// room 955 / 790, free 877 / 715), but where a few tiles have far longer lists than the others their two
+// warps set the time, on larger grids the longer the more Gaussians (aerial scene: 1200 tiles 338 / 430, 4032
+// 438 / 561, 10800 913 / 1066, 57600 4840 / 3840), and the host does not know the lists. The autotuner measures.
 // A caller who fixes only one of the two passes gets 2 for the other.
 int pick_px(int requested, int fallback) { return (requested == 1 || requested == 2 || requested == 4) ? requested : fallback; }
-int default_px(const Layout& L, bool backward) {
+int default_px(const Layout& L) {
   if (pick_px(L.fwd_px, 0) || pick_px(L.bwd_px, 0)) return 2;
-  return L.n_tiles >= (backward ? 1024 : 4000) ? 4 : 2;
+  return L.n_tiles >= 20000 ? 4 : 2;
 }
 // chunk depth: a power of two in [lo, hi], else the default
 int pick_chunk(int requested, int lo, int hi, int fallback) {

@@ -491,7 +491,7 @@ cudaError_t launch_raster_fwd_l1_bwd(const Layout& L, void* ws, float* rgb, floa
   uint64_t *ev = &st->evals, *cp = &st->composited;
   const FusedLoss F{loss.rgb_t, loss.depth_t, loss.g_rgb, loss.g_depth, at<float>(ws, L.tile_loss), &st->loss_ctr,
                     loss.d_loss};
-  const int px = pick_px(L.fwd_px, default_px(L, true));
+  const int px = pick_px(L.fwd_px, default_px(L));
   const int ch = pick_chunk(L.fwd_chunk, 64, 256, kFwdChunk);
   // the backward phase stages kBwdChunk splats per chunk (the chunk depth changes no result); at 4
   // pixels per thread, a grid that the variant without the blocks-per-SM register budget runs in
@@ -552,7 +552,7 @@ cudaError_t launch_raster_fwd(const Layout& L, void* ws, float* rgb, float* dept
   if (loss)
     F = FusedLoss{loss->rgb_t, loss->depth_t, loss->g_rgb, loss->g_depth, at<float>(ws, L.tile_loss), &st->loss_ctr,
                   loss->d_loss};
-  const int px = pick_px(L.fwd_px, default_px(L, loss != nullptr));
+  const int px = pick_px(L.fwd_px, default_px(L));
   const int ch = pick_chunk(L.fwd_chunk, 64, 256, kFwdChunk);
 #define GS_FWD(P, C, ST, LO)                                                                                  \
   launch(k_raster_fwd<P, C, ST, LO>, grid, kTilePixels / P, cap_smem(k_raster_fwd<P, C, ST, LO>, L.raster_bps), s, \
