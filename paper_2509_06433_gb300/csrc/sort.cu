@@ -10,6 +10,8 @@
 // input order; tiles are numbered by a dynamic counter and the look-back sums the counts
 // of all lower-numbered tiles. The look-back spin is bounded: past kSpinLimit polls it
 // sets GS_DEVERR_TIMEOUT and stops waiting (all writes stay inside [0, n)).
+#include <algorithm>
+
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -309,10 +311,12 @@ cudaError_t launch_onesweep(const SortArgs32& a, cudaStream_t s) { return oneswe
 cudaError_t launch_sort_prepare(const SortArgs& a, cudaStream_t s) {
   cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * 256 * a.passes, s);
   cudaMemsetAsync(a.tile_ctr, 0, sizeof(uint32_t) * kMaxSortPasses, s);
-  // (every block adds its histograms to the global ones: few blocks of many keys, more only where the reading
-  // itself takes long. Whole sort, 40-bit keys, us at 2 / 4 blocks per multiprocessor / 1024 blocks of 256 keys
-  // or more: 850k 124 / 125 / 130, 1.1M 140.3 / 140.8 / 144.7, 2.7M 254.4 / 251.3 / 253.2, 4M 329 / 322 / 323)
+  // (every block adds its histograms to the global ones: few blocks of many keys, but one per multiprocessor if
+  // the keys suffice, and more where the reading itself takes long. Whole sort, 40-bit keys, us: 50k in 49 / 196
+  // blocks 57.5 / 56.9; at 2 / 4 blocks per multiprocessor / up to 1024 blocks: 850k 124 / 125 / 130, 1.1M 140.3 /
+  // 140.8 / 144.7, 2.7M 254.4 / 251.3 / 253.2, 4M 329 / 322 / 323)
   int64_t blocks = (a.n_host + 1023) / 1024;
+  if (blocks < num_sms()) blocks = std::min<int64_t>(num_sms(), (a.n_host + 255) / 256);
   const int64_t most = (a.n_host <= 1000000 ? 2 : 4) * static_cast<int64_t>(num_sms());
   if (blocks > most) blocks = most;
   if (blocks < 1) blocks = 1;
