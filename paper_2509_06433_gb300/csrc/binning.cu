@@ -443,7 +443,10 @@ cudaError_t launch_tile_scan(const Layout& L, void* ws, cudaStream_t s) {
   if (smem > 32 * 1024) {  // (images wider than 4096 pixels)
     const cudaError_t e = cudaFuncSetAttribute(k_tile_scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                kTileSubLists * kScanRows * 1024 * 4);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // returned here: not to be found again by the process's next call
+      return e;
+    }
   }
   launch(k_tile_scan, static_cast<unsigned>(L.K * L.scan_slabs), kTileScanThreads, smem, s, L, static_cast<uint8_t*>(ws));
   return cudaGetLastError();
@@ -457,7 +460,8 @@ cudaError_t launch_bin(const Layout& L, void* ws, cudaStream_t s) {
   launch(k_sorted_counts, item_grid, kProjBlock, 0, s, L, w);
   launch(k_scan_blocks, 1, kScanThreads, 0, s, L, w);
   launch(k_item_offsets, item_grid, kProjBlock, 0, s, L, w);
-  launch_tile_scan(L, ws, s);
+  const cudaError_t e = launch_tile_scan(L, ws, s);
+  if (e != cudaSuccess) return e;  // (the emission would read item offsets and ranges that nobody wrote)
   // the emission's blocks stride over the windows of emitted pairs (their number is on the device);
   // enough blocks that a typical count takes one window per block (a block looping over several
   // windows serialises their latency-bound searches), few enough that surplus blocks cost little

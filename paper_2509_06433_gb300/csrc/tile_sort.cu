@@ -546,10 +546,14 @@ cudaError_t launch_tile_bin(const Layout& L, void* ws, cudaStream_t s) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_tile_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(sizeof(LongSmem)));
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
     ready[dev] = true;
   }
-  launch_tile_scan(L, ws, s);
+  const cudaError_t e = launch_tile_scan(L, ws, s);
+  if (e != cudaSuccess) return e;  // (the emission would write at cursors that nobody set)
   const int64_t sms = device_sms();
   // groups of whole views: a group's emission covers every projection block holding its items
   const int64_t per_view = static_cast<int64_t>(L.Tx) * L.Ty;
