@@ -230,7 +230,7 @@ GS_API gs_status_t gs_project(const gs_config_t* cfg, const gs_gaussians_t* gaus
  * and a stable onesweep radix sort of the pairs on the tile bits only. The emission indices number
  * the items' pairs in increasing item order (a) or in depth order (b). The pair count stays on the
  * device; more than pair_capacity pairs sets GS_DEVERR_PAIR_OVERFLOW and leaves every tile empty. Consumes the
- * state of the preceding gs_project on the same workspace (call it once per gs_project). */
+ * state of the preceding gs_project on the same workspace (once per gs_project; again gives the same lists). */
 GS_API gs_status_t gs_bin_sort(const gs_config_t* cfg, void* ws, size_t ws_bytes, void* stream);
 
 /* Forward compositing (render I1/I2 of Fig. 3). Per pixel, front to back over its

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(Layout L, uint8_
                                              any ? static_cast<uint32_t>(end < n ? end : n) : 0u);
     if (L.tile_sort) {
       if (end - start > static_cast<uint64_t>(kTileSortShort) && n)
-        at<uint32_t>(ws, L.long_tiles)[atomicAdd(&st->n_long, 1u)] = static_cast<uint32_t>(tg);
+        at<uint32_t>(ws, L.long_tiles)[atomicAdd(&st->n_long_next, 1u)] = static_cast<uint32_t>(tg);
     } else if (any) {
       for (int p = 0; p < L.passes; ++p)
         atomicAdd(&s_hist[p * 256 + ((static_cast<uint32_t>(tg) >> (8 * p)) & 0xffu)], static_cast<uint32_t>(end - start));

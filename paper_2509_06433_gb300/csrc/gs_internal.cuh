@@ -51,6 +51,7 @@ struct Status {
   uint32_t view_ctr;        // tile-scan blocks started
   uint32_t proj_done;       // projection blocks finished (the last one scans their live counts)
   uint32_t n_long;          // tiles whose list is longer than kTileSortShort (tile-sort binning)
+  uint32_t n_long_next;     // the same while the tile scan counts them
 };
 static_assert(sizeof(Status) <= 256, "status block");
 

@@ -99,6 +99,16 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
     st->n_live = total_live;
     st->num_pairs = static_cast<uint32_t>(overflow ? cap : total_pairs);
     if (overflow) atomicOr(&st->err, GS_DEVERR_PAIR_OVERFLOW);
+    // the tile scan is over: what it counted with starts at zero again for a repeated gs_bin_sort
+    st->n_long = st->n_long_next;
+    st->n_long_next = 0;
+    st->view_ctr = 0;
+  }
+  {
+    const int64_t slabs = static_cast<int64_t>(L.K) * L.scan_slabs;
+    uint64_t* vlb = at<uint64_t>(ws, L.view_lb);
+    for (int64_t i = slabs * b / L.n_proj_groups + threadIdx.x; i < slabs * (b + 1) / L.n_proj_groups; i += kEmitThreads)
+      vlb[i] = 0;
   }
   // the record bits of the backward pass: this block's share
   {
