@@ -68,7 +68,7 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
   while (L->proj_items < kProjItemsMax && L->KN >= static_cast<int64_t>(2 * L->proj_items) * kProjTargetBlocks)
     L->proj_items *= 2;
   L->n_proj_groups = L->KN > 0 ? (L->KN + L->proj_items - 1) / L->proj_items : 1;
-  L->item_sort_items = pick_sort_items(L->KN);
+  L->item_sort_items = pick_item_sort_items(L->KN);
   L->pair_sort_items = pick_sort_items(L->cap);
   // Binning by tile sorts or by the global radix sorts. Tile sorts from one tile per multiprocessor
   // on (a list is sorted by one block) and while the lists stay short: projection + binning of 300k
