@@ -411,8 +411,9 @@ gs_status_t gs_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int32_t key
   if (n == 0) return GS_OK;
   if (!keys || !vals || !tmp || (reinterpret_cast<uintptr_t>(tmp) % kAlign) != 0) return GS_ERR_INVALID_ARG;
   SortTmp t = sort_tmp_layout(n, pick_sort_items(n));
-  // (shorter tiles take more scratch: a buffer sized for somewhat more pairs, with the long tiles, does as well)
-  if (tmp_bytes < t.total && n > kSortLongTilesFrom) t = sort_tmp_layout(n, kSortItems);
+  // (shorter tiles take more scratch: a buffer sized for more pairs, with longer tiles, does as well)
+  for (const int items : {kSortItemsMid, kSortItems})
+    if (tmp_bytes < t.total && items > t.items) t = sort_tmp_layout(n, items);
   if (tmp_bytes < t.total) return GS_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   SortArgs a{};

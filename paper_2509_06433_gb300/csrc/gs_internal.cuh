@@ -475,13 +475,13 @@ __host__ __device__ inline int64_t sort_tiles(int64_t n, int items) {
 // Keys per thread for a sort of up to n keys: small sorts take short tiles, so that enough
 // blocks share the work.
 // keys per thread: small sorts take small tiles (more blocks, shorter per-tile latency)
-// (from kSortLongTilesFrom pairs on, gs_sort_pairs also runs in scratch that only long tiles fit)
-constexpr int64_t kSortLongTilesFrom = 600000;
-inline int pick_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 1000000 ? 8 : kSortItems); }
+// (gs_sort_pairs also runs in scratch that only longer tiles fit)
+constexpr int kSortItemsMid = 8;
+inline int pick_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 1000000 ? kSortItemsMid : kSortItems); }
 // The depth sort of the items has 32-bit keys and four passes: long tiles from 600k items on. Binning by the radix
 // sorts, us with 8 / 15 keys per thread for the items: 700k 126.2 / 128.0, 800k 138.7 / 134.1, 850k 148.2 / 142.3,
 // 990k 163.8 / 153.3 (the pairs' sort as above: 8 keys for 868k pairs 117.8, 15 keys 118.5).
-inline int pick_item_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 600000 ? 8 : kSortItems); }
+inline int pick_item_sort_items(int64_t n) { return n <= 200000 ? 4 : (n <= 600000 ? kSortItemsMid : kSortItems); }
 using SortArgs = SortArgsT<uint64_t>;
 using SortArgs32 = SortArgsT<uint32_t>;
 cudaError_t launch_onesweep(const SortArgs& a, cudaStream_t s);
