@@ -21,8 +21,9 @@
 // counts the smaller keys of its own bucket. The buckets adapt to the depths' distribution: 256
 // equal slices of the list's depth range are counted first, and a slice of n pairs is cut into the
 // largest power of two <= n buckets (a wall seen next to a near object would otherwise fall into a
-// few buckets). A list that still has a bucket of more than kMaxBucket pairs (many equal or
-// almost equal depths) is sorted by a bitonic network instead.
+// few buckets). Where all depths are equal (a floor seen straight from above), the buckets are taken
+// from the slots instead. A list that still has a bucket of more than kMaxBucket pairs (many equal
+// or almost equal depths beside others) is sorted by a bitonic network.
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -104,12 +105,8 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
     st->n_long_next = 0;
     st->view_ctr = 0;
   }
-  {
-    const int64_t slabs = static_cast<int64_t>(L.K) * L.scan_slabs;
-    uint64_t* vlb = at<uint64_t>(ws, L.view_lb);
-    for (int64_t i = slabs * b / L.n_proj_groups + threadIdx.x; i < slabs * (b + 1) / L.n_proj_groups; i += kEmitThreads)
-      vlb[i] = 0;
-  }
+  if (b == 0)
+    for (int i = threadIdx.x; i < L.K * L.scan_slabs; i += kEmitThreads) at<uint64_t>(ws, L.view_lb)[i] = 0;
   // the record bits of the backward pass: this block's share
   {
     const int64_t words = (static_cast<int64_t>(overflow ? cap : total_pairs) + 31) / 32;
@@ -233,19 +230,15 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
   pdl_trigger();
 }
 
-// Working arrays of one list's sort, in shared memory or (GLOBAL) in the list's share of scratch:
-// keys, their Gaussian ids (first the depths), the buckets' counts / ends.
-template <bool GLOBAL>
+// Working arrays of one list's sort, in shared memory: keys, their Gaussian ids (first the digits that
+// the buckets are taken from), the buckets' counts / ends (two 16-bit buckets per word).
 struct SortArrays {
   uint64_t* key;
   uint32_t* gid;
-  uint32_t* fine;  // one word per bucket (GLOBAL) or two 16-bit buckets per word
+  uint32_t* fine;
 };
 // Words of the bucket counts of n pairs: at most n + kSlices buckets.
-template <bool GLOBAL>
-__host__ __device__ constexpr uint32_t bucket_words(uint32_t n) {
-  return GLOBAL ? n + kSlices : (n + kSlices + 1) / 2;
-}
+__host__ __device__ constexpr uint32_t bucket_words(uint32_t n) { return (n + kSlices + 1) / 2; }
 struct SortShared {
   uint32_t slice[kSlices];     // pairs of each slice, then its first bucket << 5 | bucket bits
   uint32_t warp[3][32];
@@ -253,15 +246,11 @@ struct SortShared {
 };
 
 // One more pair in bucket f; returns the bucket's count before.
-template <bool GLOBAL>
 __device__ __forceinline__ uint32_t bucket_add(uint32_t* fine, uint32_t f) {
-  if (GLOBAL) return atomicAdd(&fine[f], 1u);
   const uint32_t sh = 16 * (f & 1u);
   return (atomicAdd(&fine[f >> 1], 1u << sh) >> sh) & 0xffffu;
 }
-template <bool GLOBAL>
 __device__ __forceinline__ uint32_t bucket_get(const uint32_t* fine, uint32_t f) {
-  if (GLOBAL) return __ldcg(&fine[f]);  // (global counts are changed by atomics, which pass the L1 by)
   return reinterpret_cast<const uint16_t*>(fine)[f];
 }
 
@@ -285,17 +274,16 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* tmp, uint32
   return before + excl;
 }
 
-// Sorts the n records rec[0, n) of tile `tile`; writes keys_out[i] = (tile << 32) | Gaussian id and
-// vals_out[i] = slot. All threads of the block call it.
-template <int THREADS, bool GLOBAL>
-__device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_t n, SortArrays<GLOBAL> A, SortShared& S,
-                                          uint64_t tile, uint64_t* __restrict__ keys_out,
-                                          uint32_t* __restrict__ vals_out) {
+// The digits of a record that its bucket is taken from, their least and largest, and all of them in A.gid.
+struct DigitRange {
+  uint32_t lo, hi;
+};
+template <int THREADS, bool SLOTS>
+__device__ __forceinline__ DigitRange list_digits(const uint4* rec, uint32_t n, SortArrays A, SortShared& S) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  // the depths and their range
   uint32_t lo = 0xffffffffu, hi = 0;
   for (uint32_t i = t; i < n; i += THREADS) {
-    const uint32_t d = rec[i].x;
+    const uint32_t d = SLOTS ? rec[i].y : rec[i].x;
     A.gid[i] = d;
     lo = min(lo, d);
     hi = max(hi, d);
@@ -314,6 +302,17 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
     lo = min(lo, S.warp[0][w]);
     hi = max(hi, S.warp[1][w]);
   }
+  return {lo, hi};
+}
+
+// Sorts the n records rec[0, n) of tile `tile` by their digits (the depths, or with SLOTS the slots); writes
+// keys_out[i] = (tile << 32) | Gaussian id and vals_out[i] = slot. All threads of the block call it.
+template <int THREADS, bool SLOTS>
+__device__ __forceinline__ void sort_digits(const uint4* rec, uint32_t n, DigitRange range, SortArrays A, SortShared& S,
+                                            uint64_t tile, uint64_t* __restrict__ keys_out,
+                                            uint32_t* __restrict__ vals_out) {
+  const int t = threadIdx.x, lane = t & 31;
+  const uint32_t lo = range.lo, hi = range.hi;
   const int bits = 32 - __clz(hi - lo), shift = bits > 8 ? bits - 8 : 0;
   // pairs per slice, buckets per slice
   for (uint32_t i = t; i < n; i += THREADS) atomicAdd(&S.slice[(A.gid[i] - lo) >> shift], 1u);
@@ -327,7 +326,7 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
   uint32_t n_fine;
   const uint32_t f0 = block_scan<THREADS>(nf, S.warp[2], &n_fine);
   if (t < kSlices) S.slice[t] = (f0 << 5) | fbits;
-  const uint32_t words = GLOBAL ? n_fine : (n_fine + 1) / 2;
+  const uint32_t words = (n_fine + 1) / 2;
   for (uint32_t i = t; i < words; i += THREADS) A.fine[i] = 0;
   __syncthreads();
   const uint32_t rest = (1u << shift) - 1u;  // (shift <= 24)
@@ -335,7 +334,7 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
     const uint32_t s = S.slice[(d - lo) >> shift];
     return (s >> 5) + (((d - lo) & rest) >> (shift - (s & 31u)));
   };
-  for (uint32_t i = t; i < n; i += THREADS) bucket_add<GLOBAL>(A.fine, bucket(A.gid[i]));
+  for (uint32_t i = t; i < n; i += THREADS) bucket_add(A.fine, bucket(A.gid[i]));
   __syncthreads();
   // exclusive prefix of the bucket counts (a run of consecutive words per thread)
   {
@@ -343,17 +342,15 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
     const uint32_t i0 = min(t * per, words), i1 = min(i0 + per, words);
     uint32_t sum = 0, most = 0;
     for (uint32_t i = i0; i < i1; ++i) {
-      const uint32_t c = GLOBAL ? __ldcg(&A.fine[i]) : A.fine[i];
-      const uint32_t c0 = GLOBAL ? c : c & 0xffffu, c1 = GLOBAL ? 0u : c >> 16;
+      const uint32_t c0 = A.fine[i] & 0xffffu, c1 = A.fine[i] >> 16;
       sum += c0 + c1;
       most = max(most, max(c0, c1));
     }
     uint32_t all;
     uint32_t at0 = block_scan<THREADS>(sum, S.warp[0], &all);
     for (uint32_t i = i0; i < i1; ++i) {
-      const uint32_t c = GLOBAL ? __ldcg(&A.fine[i]) : A.fine[i];
-      const uint32_t c0 = GLOBAL ? c : c & 0xffffu, c1 = GLOBAL ? 0u : c >> 16;
-      A.fine[i] = GLOBAL ? at0 : (at0 | ((at0 + c0) << 16));
+      const uint32_t c0 = A.fine[i] & 0xffffu, c1 = A.fine[i] >> 16;
+      A.fine[i] = at0 | ((at0 + c0) << 16);
       at0 += c0 + c1;
     }
     most = __reduce_max_sync(0xffffffffu, most);
@@ -363,7 +360,7 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
   // into the buckets; afterwards fine[f] is bucket f's end
   for (uint32_t i = t; i < n; i += THREADS) {
     const uint4 r = rec[i];
-    const uint32_t pos = bucket_add<GLOBAL>(A.fine, bucket(r.x));
+    const uint32_t pos = bucket_add(A.fine, bucket(SLOTS ? r.y : r.x));
     A.key[pos] = (static_cast<uint64_t>(r.x) << 32) | r.y;
     A.gid[pos] = r.z;
   }
@@ -372,8 +369,8 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
   if (S.max_bucket == 0) {
     for (uint32_t i = t; i < n; i += THREADS) {
       const uint64_t key = A.key[i];
-      const uint32_t f = bucket(static_cast<uint32_t>(key >> 32));
-      const uint32_t s = f ? bucket_get<GLOBAL>(A.fine, f - 1) : 0u, e = bucket_get<GLOBAL>(A.fine, f);
+      const uint32_t f = bucket(static_cast<uint32_t>(SLOTS ? key : key >> 32));
+      const uint32_t s = f ? bucket_get(A.fine, f - 1) : 0u, e = bucket_get(A.fine, f);
       uint32_t rank = s;
       for (uint32_t j = s; j < e; ++j) rank += A.key[j] < key ? 1u : 0u;
       keys_out[rank] = hi_word | A.gid[i];
@@ -382,14 +379,13 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
     return;
   }
   // bitonic network over the next power of two (absent keys compare as the largest)
-  uint32_t m = 1;
-  while (m < n) m <<= 1;
-  for (uint32_t k = 2; k <= m; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      for (uint32_t q = t; q < m / 2; q += THREADS) {
+  const int levels = 32 - __clz(n - 1);  // (n > kMaxBucket here)
+  for (int k = 0; k < levels; ++k) {
+    for (int j = k; j >= 0; --j) {
+      for (uint32_t q = t; q < 1u << (levels - 1); q += THREADS) {
         // the first step of a merge compares mirrored positions, so every comparison is ascending
-        const uint32_t a = (q / j) * 2 * j + (q % j);
-        const uint32_t c = (j == k >> 1) ? (q / j) * 2 * j + (2 * j - 1 - q % j) : a + j;
+        const uint32_t r = q & ((1u << j) - 1u), a = ((q >> j) << (j + 1)) + r;
+        const uint32_t c = j == k ? a + (2u << j) - 1u - 2u * r : a + (1u << j);
         if (c < n) {
           const uint64_t ka = A.key[a], kc = A.key[c];
           if (kc < ka) {
@@ -410,11 +406,32 @@ __device__ __forceinline__ void sort_list(const uint4* __restrict__ rec, uint32_
   }
 }
 
+// (A call of its own: with both digits in one loop the common lists took 1 to 2 us longer.)
+template <int THREADS>
+__device__ __noinline__ void sort_by_slot(const uint4* rec, uint32_t n, SortArrays A, SortShared& S, uint64_t tile,
+                                          uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out) {
+  const DigitRange slots = list_digits<THREADS, true>(rec, n, A, S);
+  sort_digits<THREADS, true>(rec, n, slots, A, S, tile, keys_out, vals_out);
+}
+
+// Sorts the n records rec[0, n): by depth, or by slot where all depths are equal.
+template <int THREADS>
+__device__ __forceinline__ void sort_list(const uint4* rec, uint32_t n, SortArrays A, SortShared& S, uint64_t tile,
+                                          uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out) {
+  const DigitRange depths = list_digits<THREADS, false>(rec, n, A, S);
+  if (depths.lo != depths.hi) {
+    sort_digits<THREADS, false>(rec, n, depths, A, S, tile, keys_out, vals_out);
+  } else {
+    __syncthreads();  // the warps' ranges are read
+    sort_by_slot<THREADS>(rec, n, A, S, tile, keys_out, vals_out);
+  }
+}
+
 template <int CAP>
 struct ListSmem {
   uint64_t key[CAP];
   uint32_t gid[CAP];
-  uint32_t fine[bucket_words<false>(CAP)];
+  uint32_t fine[bucket_words(CAP)];
   SortShared S;
 };
 
@@ -426,121 +443,159 @@ __global__ void __launch_bounds__(kShortThreads) k_tile_sort(Layout L, uint8_t* 
   const uint2 rg = at<uint2>(ws, L.ranges)[tile];
   const uint32_t n = rg.y - rg.x;
   if (n > 0 && n <= static_cast<uint32_t>(kTileSortShort))
-    sort_list<kShortThreads, false>(at<uint4>(ws, L.pair_grads) + rg.x, n, SortArrays<false>{M.key, M.gid, M.fine}, M.S,
+    sort_list<kShortThreads>(at<uint4>(ws, L.pair_grads) + rg.x, n, SortArrays{M.key, M.gid, M.fine}, M.S,
                                     static_cast<uint64_t>(tile), at<uint64_t>(ws, L.keys[0]) + rg.x,
                                     at<uint32_t>(ws, L.vals[0]) + rg.x);
   pdl_trigger();
 }
 
 // The lists longer than kTileSortShort, taken from the tile scan's list by a grid of resident blocks.
-// A list of more than kLongShared pairs is first cut by depth: its records go, in the order of
-// kLongSlices equal slices of its depth range, to the list's share of scratch, and runs of slices that
-// fit are sorted in shared memory one after another (a single slice that does not fit is sorted in
-// global memory). Behind the unsorted records, a list that starts at pair s owns the 32 bytes per
-// pair of pair_grads from byte 16 capacity + 32 s on: 16 n bytes of cut records, then the buckets of
-// a global sort, whose keys and ids take the place of the unsorted records.
+// A list of more than kLongShared pairs is first cut: its records go to the other record buffer in the order
+// of kLongSlices equal slices of its depth range, and runs of slices that fit are sorted in shared memory
+// one after another. A slice that does not fit (a wall among scattered depths) is cut again on its own, from
+// that buffer to the first. A segment of fewer different depths than slices is cut by depths and slots
+// written as one number, ((depth - least depth) << slot bits) | (slot - least slot). Either range loses 11
+// bits each time, so no list is cut more than seven times (32 and 30 bits). The record buffers are the 16
+// bytes per pair of pair_grads from byte 0 and from byte 16 capacity on; the third 16 bytes hold the slices
+// still to be cut. Projection and binning of 12,000 / 200,000 pairs of one tile, us: all depths equal 78 / 742
+// (932 / 18,311 when such slices went through a network of compare-exchanges in global memory), half of them
+// equal 110 / 1003 (484 / 8954), all different 82 / 784.
 struct LongSmem {
   ListSmem<kLongShared> list;
   uint32_t slice[kLongSlices];
-  uint32_t lo[kLongThreads / 32], hi[kLongThreads / 32];
+  uint32_t lo[2][kLongThreads / 32], hi[2][kLongThreads / 32];
 };
+struct Segment {  // records [start, start + n) of buffer src
+  uint32_t start, n, src;
+};
+constexpr int kSliceBits = 11;
+static_assert(kLongSlices == 1 << kSliceBits, "slices of a power-of-two width");
 
-__global__ void __launch_bounds__(kLongThreads, kLongBlocks) k_tile_sort_long(Layout L, uint8_t* __restrict__ ws) {
-  pdl_wait();
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  LongSmem& M = *reinterpret_cast<LongSmem*>(smem_raw);
-  const SortArrays<false> shared{M.list.key, M.list.gid, M.list.fine};
+// Least and largest word `w` (0 depth, 1 slot) of the records.
+__device__ __forceinline__ DigitRange word_range(const uint4* rec, uint32_t n, int w, LongSmem& M) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const uint32_t n_long = at<Status>(ws, L.status)->n_long;
-  for (uint32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
-    const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[i];
-    const uint2 rg = at<uint2>(ws, L.ranges)[tile];
-    const uint32_t n = rg.y - rg.x;
-    uint4* rec = at<uint4>(ws, L.pair_grads) + rg.x;
-    uint64_t* keys = at<uint64_t>(ws, L.keys[0]) + rg.x;
-    uint32_t* vals = at<uint32_t>(ws, L.vals[0]) + rg.x;
-    if (n <= static_cast<uint32_t>(kLongShared)) {
-      sort_list<kLongThreads, false>(rec, n, shared, M.list.S, tile, keys, vals);
-      __syncthreads();  // the next list reuses the shared arrays
-      continue;
-    }
-    uint8_t* scratch = ws + L.pair_grads + 16 * static_cast<size_t>(L.cap) + 32 * static_cast<size_t>(rg.x);
-    uint4* cut = reinterpret_cast<uint4*>(scratch);
-    uint32_t lo = 0xffffffffu, hi = 0;
-    for (uint32_t j = t; j < n; j += kLongThreads) {
-      const uint32_t d = rec[j].x;
-      lo = min(lo, d);
-      hi = max(hi, d);
-    }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (lane == 0) {
-      M.lo[warp] = lo;
-      M.hi[warp] = hi;
-    }
-    for (int s = t; s < kLongSlices; s += kLongThreads) M.slice[s] = 0;
-    __syncthreads();
+  uint32_t lo = 0xffffffffu, hi = 0;
+  for (uint32_t j = t; j < n; j += kLongThreads) {
+    const uint32_t d = reinterpret_cast<const uint32_t*>(&rec[j])[w];
+    lo = min(lo, d);
+    hi = max(hi, d);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    M.lo[w][warp] = lo;
+    M.hi[w][warp] = hi;
+  }
+  __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kLongThreads / 32; ++w) {
-      lo = min(lo, M.lo[w]);
-      hi = max(hi, M.hi[w]);
-    }
-    constexpr int kBits = 11;
-    static_assert(kLongSlices == 1 << kBits, "slices of a power-of-two width");
-    const int bits = 32 - __clz(hi - lo), shift = bits > kBits ? bits - kBits : 0;
-    for (uint32_t j = t; j < n; j += kLongThreads) atomicAdd(&M.slice[(rec[j].x - lo) >> shift], 1u);
-    __syncthreads();
-    {
-      constexpr int kPer = kLongSlices / kLongThreads;
-      uint32_t c[kPer], sum = 0, all;
+  for (int v = 0; v < kLongThreads / 32; ++v) {
+    lo = min(lo, M.lo[w][v]);
+    hi = max(hi, M.hi[w][v]);
+  }
+  return {lo, hi};
+}
+
+// Moves the n records to `cut` in the order of their slices; M.slice (zero before) then holds the slices' ends.
+template <class Slice>
+__device__ __forceinline__ void cut_by(const uint4* rec, uint4* cut, uint32_t n, LongSmem& M, Slice slice) {
+  const int t = threadIdx.x;
+  for (uint32_t j = t; j < n; j += kLongThreads) atomicAdd(&M.slice[slice(rec[j])], 1u);
+  __syncthreads();
+  {
+    constexpr int kPer = kLongSlices / kLongThreads;
+    uint32_t c[kPer], sum = 0, all;
 #pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        c[q] = M.slice[t * kPer + q];
-        sum += c[q];
-      }
-      uint32_t at0 = block_scan<kLongThreads>(sum, M.list.S.warp[0], &all);
+    for (int q = 0; q < kPer; ++q) {
+      c[q] = M.slice[t * kPer + q];
+      sum += c[q];
+    }
+    uint32_t at0 = block_scan<kLongThreads>(sum, M.list.S.warp[0], &all);
 #pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        M.slice[t * kPer + q] = at0;
-        at0 += c[q];
-      }
+    for (int q = 0; q < kPer; ++q) {
+      M.slice[t * kPer + q] = at0;
+      at0 += c[q];
     }
-    __syncthreads();
-    for (uint32_t j = t; j < n; j += kLongThreads) {
-      const uint4 r = rec[j];
-      cut[atomicAdd(&M.slice[(r.x - lo) >> shift], 1u)] = r;
-    }
-    __syncthreads();  // slice[s] is now slice s's end
+  }
+  __syncthreads();
+  for (uint32_t j = t; j < n; j += kLongThreads) {
+    const uint4 r = rec[j];
+    cut[atomicAdd(&M.slice[slice(r)], 1u)] = r;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void cut_segment(const uint4* rec, uint4* cut, uint32_t n, LongSmem& M) {
+  for (int s = threadIdx.x; s < kLongSlices; s += kLongThreads) M.slice[s] = 0;
+  const DigitRange d = word_range(rec, n, 0, M);
+  const int bits = 32 - __clz(d.hi - d.lo);
+  if (bits >= kSliceBits) {
+    const int shift = bits - kSliceBits;
+    cut_by(rec, cut, n, M, [=](const uint4& r) { return (r.x - d.lo) >> shift; });
+  } else {
+    const DigitRange s = word_range(rec, n, 1, M);
+    const int sbits = 32 - __clz(s.hi - s.lo), shift = max(bits + sbits - kSliceBits, 0);
+    cut_by(rec, cut, n, M, [=](const uint4& r) {
+      return static_cast<uint32_t>(((static_cast<uint64_t>(r.x - d.lo) << sbits) | (r.y - s.lo)) >> shift);
+    });
+  }
+}
+
+// Sorts the segment of `tile`'s list by the whole block.
+__device__ __forceinline__ void sort_segment(const Layout& L, uint8_t* __restrict__ ws, uint32_t tile, Segment seg,
+                                             LongSmem& M) {
+  uint4* const buf = at<uint4>(ws, L.pair_grads);
+  uint4* const left = buf + 2 * L.cap + seg.start;  // the slices still to be cut
+  const SortArrays shared{M.list.key, M.list.gid, M.list.fine};
+  auto in_shared = [&](uint32_t src, uint32_t start, uint32_t n) {
+    sort_list<kLongThreads>(buf + src * L.cap + start, n, shared, M.list.S, tile, at<uint64_t>(ws, L.keys[0]) + start,
+                            at<uint32_t>(ws, L.vals[0]) + start);
+    __syncthreads();  // the next piece reuses the arrays
+  };
+  if (seg.n <= static_cast<uint32_t>(kLongShared)) {
+    in_shared(seg.src, seg.start, seg.n);
+    return;
+  }
+  for (int n_left = 0;;) {
+    const uint32_t other = seg.src ^ 1u;
+    cut_segment(buf + seg.src * L.cap + seg.start, buf + other * L.cap + seg.start, seg.n, M);
     uint32_t start = 0;
-    for (int s0 = 0; s0 < kLongSlices && start < n;) {
+    for (int s0 = 0; s0 < kLongSlices && start < seg.n;) {
       int a = s0, b = kLongSlices;  // the most slices [s0, a) whose records fit
       while (a < b) {
         const int mid = (a + b + 1) / 2;
         if (M.slice[mid - 1] - start <= static_cast<uint32_t>(kLongShared)) a = mid; else b = mid - 1;
       }
-      if (a > s0) {
-        const uint32_t m = M.slice[a - 1] - start;
-        if (m > 0) sort_list<kLongThreads, false>(cut + start, m, shared, M.list.S, tile, keys + start, vals + start);
-        start += m;
-        s0 = a;
-      } else {
-        const uint32_t m = M.slice[s0] - start;
-        uint64_t* key = reinterpret_cast<uint64_t*>(rec);
-        sort_list<kLongThreads, true>(cut + start, m,
-                                      SortArrays<true>{key, reinterpret_cast<uint32_t*>(key + n),
-                                                       reinterpret_cast<uint32_t*>(scratch + 16 * static_cast<size_t>(n))},
-                                      M.list.S, tile, keys + start, vals + start);
-        start += m;
-        ++s0;
+      const bool fits = a > s0;
+      a = fits ? a : s0 + 1;
+      const uint32_t m = M.slice[a - 1] - start;
+      if (fits && m > 0) in_shared(other, seg.start + start, m);
+      if (!fits) {
+        if (threadIdx.x == 0) left[n_left] = make_uint4(seg.start + start, m, other, 0u);
+        ++n_left;
       }
-      __syncthreads();  // the next piece reuses the arrays
+      start += m;
+      s0 = a;
     }
+    __syncthreads();  // the last slices and the list of those left are read and written
+    if (n_left == 0) return;
+    const uint4 next = left[--n_left];
+    seg = Segment{next.x, next.y, next.z};
+  }
+}
+
+__global__ void __launch_bounds__(kLongThreads, kLongBlocks) k_tile_sort_long(Layout L, uint8_t* __restrict__ ws) {
+  pdl_wait();
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  LongSmem& M = *reinterpret_cast<LongSmem*>(smem_raw);
+  const uint32_t n_long = at<Status>(ws, L.status)->n_long;
+  for (uint32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
+    const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[i];
+    const uint2 rg = at<uint2>(ws, L.ranges)[tile];
+    sort_segment(L, ws, tile, Segment{rg.x, rg.y - rg.x, 0u}, M);
   }
   pdl_trigger();
 }
 static_assert(kLongShared < 65536, "16-bit bucket counts in shared memory");
-static_assert(4ull * bucket_words<true>(kLongShared + 1) <= 16ull * (kLongShared + 1), "a global sort's buckets fit");
-static_assert(kPairGradStride * sizeof(float) >= 48, "pair_grads holds the unsorted records and the scratch");
+static_assert(kPairGradStride * sizeof(float) >= 48, "pair_grads holds both record buffers and the list of slices");
 
 }  // namespace
 

@@ -50,3 +50,28 @@ def test_one_list(n, depths):
     params, cam = heap(n, DEPTHS[depths])
     r = _check(params, cam, W, H, cap=max(n, 64))
     assert r.layout.bin_sort_launches == 4
+
+
+def bin_ms(n, depths):
+    """Median device time of gs_bin_sort for one list of n pairs."""
+    from tests.gpu_common import gpu_render, torch_mods
+    torch, api = torch_mods()
+    params, cam = heap(n, DEPTHS[depths])
+    r, g, cams, _ = gpu_render(params, cam, W, H, cap=n)
+    times = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        api.gs_project(r.cfg, g, cams, r.ws)
+        a.record()
+        api.gs_bin_sort(r.cfg, r.ws)
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return float(np.median(times))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("depths", ["equal", "wall", "floors"])
+def test_equal_depths_cost_little_more(depths):
+    # (20000 pairs through a network of compare-exchanges of one block: more than 15 times as long)
+    assert bin_ms(20000, depths) < 4.0 * bin_ms(20000, "spread")
