@@ -75,7 +75,8 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
   // Gaussians on planes at 640x480 (250 per tile, lists of 2018) takes 134 us against 198 by the
   // radix sorts, 600k 283 against 318, 1M (833 per tile, lists of 6723) 473 against 465, 2M 941
   // against 850; Gaussians in free space (13 pairs each), 767 per tile (lists of 5142) 494 against 535,
-  // 1011 (lists of 12972) 1029 against 925.
+  // 1011 (lists of 12972) 1029 against 925. The host does not know the lists: a view that crowds into few
+  // tiles keeps the tile sorts, whose long lists are then shared out (k_tile_sort_long has the times).
   L->tile_sort = L->n_tiles >= kTileSortMinTiles && L->N > 0 && L->N <= kTileSortMaxItems &&
                  L->KN <= kTileSortMaxDensity * L->n_tiles;
   L->sort_groups = static_cast<int>((L->KN + kTileSortGroupItems - 1) / kTileSortGroupItems);
@@ -150,6 +151,8 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
     L->block_pairs = take(static_cast<size_t>(L->n_proj_groups) * 4);
     L->tile_cursor = take(static_cast<size_t>(L->n_tiles) * kTileSubLists * kCursorStride * 4);
     L->long_tiles = take(static_cast<size_t>(L->n_tiles) * 4);
+    L->max_tasks = static_cast<uint32_t>(cap / 32 + 64);  // (see kChunk)
+    L->tasks = take(static_cast<size_t>(L->max_tasks) * 16);
   }
   L->live_mask = take((KN + 31) / 32 * 4);
   L->live_wpre = take((KN + 31) / 32 * 4);

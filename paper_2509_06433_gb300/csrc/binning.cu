@@ -283,8 +283,10 @@ __global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(Layout L, uint8_
     at<uint2>(ws, L.ranges)[tg] = make_uint2(any ? static_cast<uint32_t>(start < n ? start : n) : 0u,
                                              any ? static_cast<uint32_t>(end < n ? end : n) : 0u);
     if (L.tile_sort) {
-      if (end - start > static_cast<uint64_t>(kTileSortShort) && n)
+      if (end - start > static_cast<uint64_t>(kTileSortShort) && n) {
         at<uint32_t>(ws, L.long_tiles)[atomicAdd(&st->n_long_next, 1u)] = static_cast<uint32_t>(tg);
+        if (end - start > static_cast<uint64_t>(kTileSortGiant)) st->giant = 1;
+      }
     } else if (any) {
       for (int p = 0; p < L.passes; ++p)
         atomicAdd(&s_hist[p * 256 + ((static_cast<uint32_t>(tg) >> (8 * p)) & 0xffu)], static_cast<uint32_t>(end - start));

@@ -34,6 +34,7 @@ constexpr int kCursorStride = 8;        // u32 between two cursors: one 32-byte 
 constexpr int kTileSortMaxDensity = 800;  // Gaussians per tile of a view (see make_layout)
 constexpr int64_t kTileSortMaxItems = 1 << 25;  // most Gaussians (so list entries; 27-bit bucket numbers)
 constexpr int kTileSortShort = 2048;    // longest list sorted by a short-list block
+constexpr int kTileSortGiant = 16384;   // longest list that one block cuts
 constexpr int kTileSortGroupItems = 6400000;  // (view, Gaussian) items per emission / sort launch
 constexpr uint32_t kSpinLimit = 1u << 21;  // bounded decoupled look-back (about a second of polling)
 
@@ -52,6 +53,9 @@ struct Status {
   uint32_t proj_done;       // projection blocks finished (the last one scans their live counts)
   uint32_t n_long;          // tiles whose list is longer than kTileSortShort (tile-sort binning)
   uint32_t n_long_next;     // the same while the tile scan counts them
+  uint32_t giant;           // whether a list is longer than kTileSortGiant
+  uint32_t task_next, task_end;  // the long lists' tasks: taken, given out
+  int32_t task_left;        // tasks given out and not done, less the done lists
 };
 static_assert(sizeof(Status) <= 256, "status block");
 
@@ -131,15 +135,17 @@ struct Layout {
   //   tile_cursor u32 [kTileSubLists][n_tiles][kCursorStride]: next free pair of each tile's
   //              sub-lists (entry 0)
   //   long_tiles  u32 [n_tiles]: the tiles with lists longer than kTileSortShort
+  //   tasks       uint4 [max_tasks]: what the blocks of k_tile_sort_long give one another to do
   // The unsorted lists are uint4 (depth bits, slot, Gaussian id, -) in the first 16 pair_capacity
   // bytes of pair_grads, which holds nothing before the backward; the rest of it is scratch of
-  // the longest lists' sorts.
+  // the long lists' sorts.
   bool tile_sort;
   int sort_groups;          // launches the views are split over (emission, sort)
   int sorted;               // buffer (keys[], vals[]) holding the sorted pairs
   size_t zero_bytes;        // the buffers from `status` on that start at zero, cleared together
   int scan_slabs;           // blocks per view of the tile scan (kScanRows tile rows each)
-  size_t stage_ell, stage_meta, surv_blocks, block_pairs, super_pairs, super_live, tile_cursor, long_tiles;
+  size_t stage_ell, stage_meta, surv_blocks, block_pairs, super_pairs, super_live, tile_cursor, long_tiles, tasks;
+  uint32_t max_tasks;
   size_t total;
 };
 

@@ -3,7 +3,8 @@
 //   k_tile_scan (binning.cu)  per-tile pair counts -> ranges, sub-lists, long tiles
 //   k_tile_emit               compaction of the live items; one unsorted record per pair
 //   k_tile_sort               lists of up to kTileSortShort pairs, in shared memory
-//   k_tile_sort_long          longer lists, cut by depth into pieces that fit in shared memory
+//   k_tile_sort_long          longer lists, cut by depth into pieces that fit in shared memory; the
+//                             longest by many blocks at once
 //
 // Order: a tile's list in (depth bits, k N + g) order, as a stable sort of ((tile << 32) | depth)
 // keys emitted in (k, g) order leaves it. A pair's slot (emission index) is its item's first pair
@@ -38,14 +39,21 @@ constexpr int kLongSlices = 2048;  // depth slices a longer one is cut into
 constexpr uint32_t kMaxBucket = 64;
 constexpr int kSlices = 256;
 
+// Most tasks that the long lists of so many pairs give out (see kChunk).
+__device__ __forceinline__ uint32_t task_bound(const Layout& L, uint64_t pairs) {
+  return min(L.max_tasks, static_cast<uint32_t>(pairs / 32 + 64));
+}
+
 // One block per projection block: compacts its live items (in item order) and writes one record
 // (depth bits, slot, Gaussian id) per pair at the next free place of its tile's sub-list: the tile
 // scan has split every list between the projection blocks b with the same b % kTileSubLists. The
 // rate is set by the cursors' atomics, about one per 30 cycles on one address and fewer when the
 // cursors of neighbouring tiles share a 32-byte sector, so that the fullest tile decides: one sector
-// per cursor and four cursors per tile. The rows of a warp's items are numbered consecutively and examined one per lane (row_span gives the same
-// tiles as in the projection), then the pairs of those 32 rows are numbered consecutively and
-// written one per lane, four rounds in flight, so that tall or wide items do not idle the warp.
+// per cursor and four cursors per tile. The rows of a warp's items are numbered consecutively and
+// examined one per lane (row_span gives the same tiles as in the projection), then the pairs of those
+// 32 rows are numbered consecutively and written one per lane, four rounds in flight, so that tall
+// or wide items do not idle the warp. (One atomic per tile and warp where a view crowds into few tiles saves
+// 0.3 of 8 ms at 2M pairs of one tile and costs 10 of 108 us of binning at 2M spread over 3600: not built.)
 __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t* __restrict__ ws, int64_t block0) {
   pdl_wait();
   constexpr int kWarps = kEmitThreads / 32;
@@ -104,9 +112,16 @@ __global__ void __launch_bounds__(kEmitThreads, 4) k_tile_emit(Layout L, uint8_t
     st->n_long = st->n_long_next;
     st->n_long_next = 0;
     st->view_ctr = 0;
+    st->task_next = st->task_end = 0;
+    st->task_left = 0;
   }
   if (b == 0)
     for (int i = threadIdx.x; i < L.K * L.scan_slabs; i += kEmitThreads) at<uint64_t>(ws, L.view_lb)[i] = 0;
+  if (st->giant) {  // no task of the long lists is written yet: this block's share
+    const int64_t n = task_bound(L, total_pairs);
+    for (int64_t i = n * b / L.n_proj_groups + threadIdx.x; i < n * (b + 1) / L.n_proj_groups; i += kEmitThreads)
+      at<uint4>(ws, L.tasks)[i].x = 0u;  // (kNoTask)
+  }
   // the record bits of the backward pass: this block's share
   {
     const int64_t words = (static_cast<int64_t>(overflow ? cap : total_pairs) + 31) / 32;
@@ -464,6 +479,8 @@ struct LongSmem {
   ListSmem<kLongShared> list;
   uint32_t slice[kLongSlices];
   uint32_t lo[2][kLongThreads / 32], hi[2][kLongThreads / 32];
+  uint4 task;
+  uint32_t word;  // one value for the whole block
 };
 struct Segment {  // records [start, start + n) of buffer src
   uint32_t start, n, src;
@@ -495,27 +512,51 @@ __device__ __forceinline__ DigitRange word_range(const uint4* rec, uint32_t n, i
   return {lo, hi};
 }
 
+// The slice of a record: of its depth, or of depth and slot as one number.
+struct Slicing {
+  uint32_t depth0, slot0;
+  int slot_bits, shift;
+  __device__ __forceinline__ uint32_t operator()(const uint4& r) const {
+    uint64_t v = static_cast<uint64_t>(r.x - depth0) << slot_bits;
+    if (slot_bits) v |= r.y - slot0;
+    return static_cast<uint32_t>(v >> shift);
+  }
+};
+__device__ __forceinline__ int depth_bits(DigitRange d) { return 32 - __clz(d.hi - d.lo); }
+__device__ __forceinline__ Slicing depth_slices(DigitRange d) { return {d.lo, 0u, 0, depth_bits(d) - kSliceBits}; }
+__device__ __forceinline__ Slicing depth_slot_slices(DigitRange d, DigitRange s) {
+  const int sbits = 32 - __clz(s.hi - s.lo);
+  return {d.lo, s.lo, sbits, max(depth_bits(d) + sbits - kSliceBits, 0)};
+}
+
+// Exclusive prefix of M.slice.
+__device__ __forceinline__ void scan_slices(LongSmem& M) {
+  constexpr int kPer = kLongSlices / kLongThreads;
+  const int t = threadIdx.x;
+  uint32_t c[kPer], sum = 0, all;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    c[q] = M.slice[t * kPer + q];
+    sum += c[q];
+  }
+  uint32_t at0 = block_scan<kLongThreads>(sum, M.list.S.warp[0], &all);
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    M.slice[t * kPer + q] = at0;
+    at0 += c[q];
+  }
+}
+__device__ __forceinline__ void clear_slices(LongSmem& M) {
+  for (int s = threadIdx.x; s < kLongSlices; s += kLongThreads) M.slice[s] = 0;
+}
+
 // Moves the n records to `cut` in the order of their slices; M.slice (zero before) then holds the slices' ends.
 template <class Slice>
 __device__ __forceinline__ void cut_by(const uint4* rec, uint4* cut, uint32_t n, LongSmem& M, Slice slice) {
   const int t = threadIdx.x;
   for (uint32_t j = t; j < n; j += kLongThreads) atomicAdd(&M.slice[slice(rec[j])], 1u);
   __syncthreads();
-  {
-    constexpr int kPer = kLongSlices / kLongThreads;
-    uint32_t c[kPer], sum = 0, all;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      c[q] = M.slice[t * kPer + q];
-      sum += c[q];
-    }
-    uint32_t at0 = block_scan<kLongThreads>(sum, M.list.S.warp[0], &all);
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      M.slice[t * kPer + q] = at0;
-      at0 += c[q];
-    }
-  }
+  scan_slices(M);
   __syncthreads();
   for (uint32_t j = t; j < n; j += kLongThreads) {
     const uint4 r = rec[j];
@@ -524,18 +565,13 @@ __device__ __forceinline__ void cut_by(const uint4* rec, uint4* cut, uint32_t n,
   __syncthreads();
 }
 __device__ __forceinline__ void cut_segment(const uint4* rec, uint4* cut, uint32_t n, LongSmem& M) {
-  for (int s = threadIdx.x; s < kLongSlices; s += kLongThreads) M.slice[s] = 0;
+  clear_slices(M);
   const DigitRange d = word_range(rec, n, 0, M);
-  const int bits = 32 - __clz(d.hi - d.lo);
-  if (bits >= kSliceBits) {
-    const int shift = bits - kSliceBits;
+  if (depth_bits(d) >= kSliceBits) {
+    const int shift = depth_bits(d) - kSliceBits;  // (written out: it is the common one)
     cut_by(rec, cut, n, M, [=](const uint4& r) { return (r.x - d.lo) >> shift; });
   } else {
-    const DigitRange s = word_range(rec, n, 1, M);
-    const int sbits = 32 - __clz(s.hi - s.lo), shift = max(bits + sbits - kSliceBits, 0);
-    cut_by(rec, cut, n, M, [=](const uint4& r) {
-      return static_cast<uint32_t>(((static_cast<uint64_t>(r.x - d.lo) << sbits) | (r.y - s.lo)) >> shift);
-    });
+    cut_by(rec, cut, n, M, depth_slot_slices(d, word_range(rec, n, 1, M)));
   }
 }
 
@@ -582,15 +618,240 @@ __device__ __forceinline__ void sort_segment(const Layout& L, uint8_t* __restric
   }
 }
 
+// Segments of more than kTileSortGiant records (a map seen from afar, all of it in a few tiles) are cut by many
+// blocks: in chunks of kChunk records they take the ranges, count the slices and move the records, one phase
+// after the other, and what comes out are segments again. All of it goes through one list of tasks that the
+// blocks take in turn. The last block to finish a phase gives out the next one's tasks, so no block waits for
+// work that another has yet to start, whichever of them are resident; a block without a task waits until there
+// is one or none is left. Tasks: per level 3 n / kChunk + 3 chunks and 2 (2 n / kLongShared + 1) segments of a
+// segment of n > kTileSortGiant, at most 0.0022 n, and at most seven levels: less than capacity / 32.
+// Projection and binning, us, by one block per list / by many (by the global radix sorts): all pairs in one tile
+// 50k 222 / 97 (81), 200k 784 / 135 (119), 800k 3147 / 284 (227), 2M 8113 / 627 (435; the cursors' atomics are
+// 0.3 ms of it); 2M in 16 tiles 829 / 348 (483). Lists of 16k are as fast either way: 64 of them 215 / 223,
+// one of 12k 80 / 83; chunks of 8192 records 90 and 229.
+constexpr int kChunk = 4096;
+constexpr int kPieceStep = kLongShared / 2;
+enum TaskKind : uint32_t { kNoTask, kSegmentTask, kRangeTask, kCountTask, kMoveTask };
+// A task: kind | source buffer << 8, tile, the segment's start, its records (kSegmentTask) or the chunk's number.
+__device__ __forceinline__ uint4 make_task(TaskKind kind, uint32_t src, uint32_t tile, uint32_t start, uint32_t n) {
+  return make_uint4(kind | src << 8, tile, start, n);
+}
+// What the blocks that cut a giant segment share, in the third record buffer from the segment's start on.
+struct Giant {
+  uint32_t n, lo[2], hi[2], done[3];
+  uint32_t slice[kLongSlices];
+};
+static_assert(sizeof(Giant) <= 16 * kTileSortGiant, "fits in the segment's part of the third buffer");
+
+__device__ __forceinline__ uint32_t load_relaxed(const uint32_t* p) { return *const_cast<const volatile uint32_t*>(p); }
+
+// Gives out the threads' tasks (at most two each, the first n of own). All threads of the block call it; what they
+// wrote before is seen by whoever takes a task. A task's first word, its kind, is written last and by itself.
+__device__ __forceinline__ void give_out(const Layout& L, uint8_t* __restrict__ ws, const uint4 (&own)[2], uint32_t n,
+                                         LongSmem& M) {
+  Status* st = at<Status>(ws, L.status);
+  uint32_t total;
+  const uint32_t mine = block_scan<kLongThreads>(n, M.list.S.warp[1], &total);
+  __threadfence();
+  if (threadIdx.x == 0) {
+    atomicAdd(&st->task_left, static_cast<int32_t>(total));
+    M.word = atomicAdd(&st->task_end, total);
+  }
+  __syncthreads();
+  const uint32_t first = M.word + mine;
+  if (n && first + n <= task_bound(L, st->total_pairs)) {
+    uint4* task = at<uint4>(ws, L.tasks) + first;
+    for (uint32_t i = 0; i < n; ++i) {
+      task[i].y = own[i].y;
+      task[i].z = own[i].z;
+      task[i].w = own[i].w;
+    }
+    __threadfence();
+    for (uint32_t i = 0; i < n; ++i) *const_cast<volatile uint32_t*>(&task[i].x) = own[i].x;
+  } else if (n) {  // (never, by the bound; whoever waits for it gives up too)
+    atomicOr(&st->err, GS_DEVERR_TIMEOUT);
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void give_out_chunks(const Layout& L, uint8_t* __restrict__ ws, TaskKind kind, uint32_t src,
+                                                uint32_t tile, uint32_t start, uint32_t n, LongSmem& M) {
+  const uint32_t chunks = (n + kChunk - 1) / kChunk;
+  for (uint32_t c0 = 0; c0 < chunks; c0 += kLongThreads) {
+    const uint32_t c = c0 + threadIdx.x;
+    const uint4 own[2] = {make_task(kind, src, tile, start, c), make_uint4(0, 0, 0, 0)};
+    give_out(L, ws, own, c < chunks ? 1u : 0u, M);
+  }
+}
+
+// Whether this block is the last to finish `done`'s phase; it then sees what the others wrote.
+__device__ __forceinline__ bool last_of(uint32_t* done, uint32_t chunks, LongSmem& M) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    M.word = atomicAdd(done, 1u) == chunks - 1 ? 1u : 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  const bool last = M.word != 0;
+  __syncthreads();
+  return last;
+}
+
+__device__ __forceinline__ void run_task(const Layout& L, uint8_t* __restrict__ ws, uint4 task, LongSmem& M) {
+  const int t = threadIdx.x;
+  const uint32_t kind = task.x & 0xffu, src = task.x >> 8, tile = task.y, start = task.z;
+  uint4* const buf = at<uint4>(ws, L.pair_grads);
+  Giant* const G = reinterpret_cast<Giant*>(buf + 2 * L.cap + start);
+  if (kind == kSegmentTask) {
+    const uint32_t n = task.w;
+    if (n <= static_cast<uint32_t>(kTileSortGiant)) {
+      sort_segment(L, ws, tile, Segment{start, n, src}, M);
+      return;
+    }
+    for (int s = t; s < kLongSlices; s += kLongThreads) G->slice[s] = 0;
+    if (t < 3) G->done[t] = 0;
+    if (t < 2) {
+      G->lo[t] = 0xffffffffu;
+      G->hi[t] = 0;
+    }
+    if (t == 0) G->n = n;
+    give_out_chunks(L, ws, kRangeTask, src, tile, start, n, M);
+    return;
+  }
+  const uint32_t n = __ldcg(&G->n), chunks = (n + kChunk - 1) / kChunk, first = task.w * kChunk;
+  const uint32_t m = min(n - first, static_cast<uint32_t>(kChunk));
+  const uint4* rec = buf + src * L.cap + start + first;
+  if (kind == kRangeTask) {
+    for (int w = 0; w < 2; ++w) {
+      const DigitRange r = word_range(rec, m, w, M);
+      if (t == 0) {
+        atomicMin(&G->lo[w], r.lo);
+        atomicMax(&G->hi[w], r.hi);
+      }
+    }
+    if (last_of(&G->done[0], chunks, M)) give_out_chunks(L, ws, kCountTask, src, tile, start, n, M);
+    return;
+  }
+  const DigitRange d{__ldcg(&G->lo[0]), __ldcg(&G->hi[0])};
+  const Slicing slice = depth_bits(d) >= kSliceBits ? depth_slices(d)
+                                                    : depth_slot_slices(d, DigitRange{__ldcg(&G->lo[1]), __ldcg(&G->hi[1])});
+  clear_slices(M);
+  __syncthreads();
+  for (uint32_t j = t; j < m; j += kLongThreads) atomicAdd(&M.slice[slice(rec[j])], 1u);
+  __syncthreads();
+  if (kind == kCountTask) {
+    for (int s = t; s < kLongSlices; s += kLongThreads)
+      if (M.slice[s]) atomicAdd(&G->slice[s], M.slice[s]);
+    if (!last_of(&G->done[1], chunks, M)) return;
+    for (int s = t; s < kLongSlices; s += kLongThreads) M.slice[s] = __ldcg(&G->slice[s]);
+    __syncthreads();
+    scan_slices(M);
+    __syncthreads();
+    for (int s = t; s < kLongSlices; s += kLongThreads) G->slice[s] = M.slice[s];
+    give_out_chunks(L, ws, kMoveTask, src, tile, start, n, M);
+    return;
+  }
+  // kMoveTask: places for the chunk's records of each slice, then the records
+  uint4* cut = buf + (src ^ 1u) * L.cap + start;
+  for (int s = t; s < kLongSlices; s += kLongThreads)
+    if (M.slice[s]) M.slice[s] = atomicAdd(&G->slice[s], M.slice[s]);
+  __syncthreads();
+  for (uint32_t j = t; j < m; j += kLongThreads) {
+    const uint4 r = rec[j];
+    cut[atomicAdd(&M.slice[slice(r)], 1u)] = r;
+  }
+  if (!last_of(&G->done[2], chunks, M)) return;
+  // the slices' ends; piece j is the run of slices that begin in [j, j + 1) kPieceStep, its last slice on its own
+  // when the run does not fit in shared memory
+  for (int s = t; s < kLongSlices; s += kLongThreads) M.slice[s] = __ldcg(&G->slice[s]);
+  __syncthreads();
+  auto begin = [&](int s) { return s ? M.slice[s - 1] : 0u; };
+  auto first_from = [&](uint32_t x) {  // the first slice that begins at x or later, kLongSlices if none does
+    int a = 0, b = kLongSlices;
+    while (a < b) {
+      const int mid = (a + b) / 2;
+      if (begin(mid) >= x) b = mid; else a = mid + 1;
+    }
+    return a;
+  };
+  for (uint32_t j0 = 0; j0 * kPieceStep < n; j0 += kLongThreads) {
+    const uint32_t x = (j0 + t) * kPieceStep;
+    uint4 own[2];
+    uint32_t n_own = 0;
+    if (x < n) {
+      const int a = first_from(x), b = first_from(x + kPieceStep);
+      const uint32_t p0 = begin(a), p1 = begin(b), last = b > a ? begin(b - 1) : p0;
+      const bool fits = p1 - p0 <= static_cast<uint32_t>(kLongShared);
+      const uint32_t mid = fits ? p1 : last;
+      if (mid > p0) own[n_own++] = make_task(kSegmentTask, src ^ 1u, tile, start + p0, mid - p0);
+      if (p1 > mid) own[n_own++] = make_task(kSegmentTask, src ^ 1u, tile, start + mid, p1 - mid);
+    }
+    give_out(L, ws, own, n_own, M);
+  }
+}
+
+// The lists as the first tasks, then those given out on the way.
+__device__ __noinline__ void run_tasks(const Layout& L, uint8_t* __restrict__ ws, LongSmem& M) {
+  Status* st = at<Status>(ws, L.status);
+  const uint32_t n_long = st->n_long;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      const uint32_t k = atomicAdd(&st->task_next, 1u);
+      uint4 task = make_uint4(kNoTask, 0, 0, 0);
+      if (k < n_long) {
+        const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[k];
+        const uint2 rg = at<uint2>(ws, L.ranges)[tile];
+        task = make_task(kSegmentTask, 0, tile, rg.x, rg.y - rg.x);
+      } else {
+        const uint32_t i = k - n_long;
+        const uint4* given = at<uint4>(ws, L.tasks) + i;
+        const bool exists = i < task_bound(L, st->total_pairs);
+        // (no fence while waiting: it would empty the L1 of the blocks that work on the same multiprocessor)
+        for (uint32_t spins = 0;; ++spins) {
+          uint32_t x = exists ? load_relaxed(&given->x) : 0u;
+          const bool over = !x && n_long + load_relaxed(reinterpret_cast<const uint32_t*>(&st->task_left)) == 0;
+          if (over) {  // tasks that were given out before the last one was done are seen now
+            __threadfence();
+            x = exists ? load_relaxed(&given->x) : 0u;
+          }
+          if (x) {
+            __threadfence();
+            task = make_uint4(x, __ldcg(&given->y), __ldcg(&given->z), __ldcg(&given->w));
+          }
+          if (x || over) break;
+          if (spins == kSpinLimit / 4) {
+            atomicOr(&st->err, GS_DEVERR_TIMEOUT);
+            break;
+          }
+          __nanosleep(min(100u << min(spins, 4u), 1000u));
+        }
+      }
+      M.task = task;
+    }
+    __syncthreads();
+    const uint4 task = M.task;
+    if ((task.x & 0xffu) == kNoTask) return;
+    run_task(L, ws, task, M);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(&st->task_left, -1);
+  }
+}
+
 __global__ void __launch_bounds__(kLongThreads, kLongBlocks) k_tile_sort_long(Layout L, uint8_t* __restrict__ ws) {
   pdl_wait();
   extern __shared__ __align__(16) uint8_t smem_raw[];
   LongSmem& M = *reinterpret_cast<LongSmem*>(smem_raw);
-  const uint32_t n_long = at<Status>(ws, L.status)->n_long;
-  for (uint32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
-    const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[i];
-    const uint2 rg = at<uint2>(ws, L.ranges)[tile];
-    sort_segment(L, ws, tile, Segment{rg.x, rg.y - rg.x, 0u}, M);
+  const Status* st = at<Status>(ws, L.status);
+  if (st->giant) {
+    run_tasks(L, ws, M);
+  } else {
+    const uint32_t n_long = st->n_long;
+    for (uint32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
+      const uint32_t tile = at<uint32_t>(ws, L.long_tiles)[i];
+      const uint2 rg = at<uint2>(ws, L.ranges)[tile];
+      sort_segment(L, ws, tile, Segment{rg.x, rg.y - rg.x, 0u}, M);
+    }
   }
   pdl_trigger();
 }

@@ -31,7 +31,7 @@ DEPTHS = {
     # most depths within a few hundred representable values, the rest far away
     "cluster": lambda rng, n: np.where(rng.random(n) < 0.9, 4.0 + rng.integers(0, 300, n) * 4.8e-7, rng.uniform(2.0, 9.0, n)),
 }
-LENGTHS = [1, 64, 65, 2047, 2048, 2049, 4607, 4608, 4609, 9216, 9217]
+LENGTHS = [1, 64, 65, 2047, 2048, 2049, 4607, 4608, 4609, 9216, 9217, 16384, 16385, 70000]
 
 
 def test_the_lists_have_the_lengths_they_are_named_after():
@@ -75,3 +75,9 @@ def bin_ms(n, depths):
 def test_equal_depths_cost_little_more(depths):
     # (20000 pairs through a network of compare-exchanges of one block: more than 15 times as long)
     assert bin_ms(20000, depths) < 4.0 * bin_ms(20000, "spread")
+
+
+@pytest.mark.gpu
+def test_many_blocks_share_a_giant_list():
+    # (one block alone: more than 12 times as long)
+    assert bin_ms(300000, "spread") < 5.0 * bin_ms(15000, "spread")
