@@ -144,6 +144,7 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
     L->emit_first = take(static_cast<size_t>(L->n_emit_blocks) * 4);
     L->emit_last = take(static_cast<size_t>(L->n_emit_blocks) * 4);
     L->live_rows = take(KN * 8);
+    L->live_bases = take(static_cast<size_t>(L->n_proj_groups) * 4);
   } else {
     L->stage_ell = take(KN * 32);
     L->stage_meta = take(KN * 16);
@@ -160,7 +161,6 @@ bool make_layout(const gs_config_t* cfg, Layout* L) {
   L->live_count = take(KN * 4);
   L->live_off = take(KN * 4);
   L->live_blocks = take(static_cast<size_t>(L->n_proj_groups) * 4);
-  L->live_bases = take(static_cast<size_t>(L->n_proj_groups) * 4);
   L->item_partials = take(KN * 16 * 4);
   L->total = o;
   return true;

@@ -117,7 +117,7 @@ struct Layout {
   //   live_count u32 [KN]: tiles emitted by each of them
   //   live_rows  uint2 [KN]: their row-span table entries (first entry, number of entries)
   //   live_off   u32 [KN]: their first pair index (emission order), clamped to the capacity
-  //   live_blocks, live_bases  u32 [n_proj_groups]: live items of each projection block, and
+  //   live_blocks, live_bases  u32 [n_proj_groups]: live items of each projection block, and (radix sorts)
   //              the block's first position among all live items (scanned by the last block)
   //   view_lb    u64 [K * scan_slabs]: look-back status of the tile scan's blocks
   //   item_partials float [KN][16]: the projection backward's per-live-item partial gradients

@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_project(Layout L, GaussPtrs
 // pass: it counts each item's emitted tiles and adds the spans to the block's copy of the span grid.
 // Bound by instruction issue (52..66% of the slots) and, at 28 of 64 warps, latency. Storage types fixed
 // at compile time, cameras in shared memory, survivors listed instead of searched for, and no barrier
-// per 256 survivors: 2 views of 1M Gaussians 110 -> 87 us, 8 of 250k 107 -> 86, 2 of 100k 28 -> 25
+// per 256 survivors: one view of 2M Gaussians 110 -> 87 us, 8 of 500k 107 -> 86, 2 of 100k 28 -> 25
 // (device time of the kernel alone). 3 blocks per SM without the 64-register limit 100 us, 5 blocks
 // with spills 82 / 88; blocks of half the items 92 / 96 (clearing and flushing the grid).
 template <int DT, bool MF32>

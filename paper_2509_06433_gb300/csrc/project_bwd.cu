@@ -123,15 +123,16 @@ constexpr int kPartial = 16;
 // compact order of the live items (increasing k N + g): sums the item's pair records in slot
 // order (warp-cooperatively for items with many pairs), applies the chain rule of the view's
 // projection, writes the item's partial (when parameter gradients are wanted) and sums the
-// items' pose gradients per view. The blocks stride over chunks of kPoseBlock live items; a chunk's items are in view order, so each view k present in chunk c gets the chunk's sum in slot
-// c + k of pose_partials (unique: a later chunk's first view is at least this chunk's last), which
-// k_pose_reduce sums over the view's chunks in order.
+// items' pose gradients per view. The blocks stride over chunks of kPoseBlock live items; a chunk's
+// items are in view order, so each view k present in chunk c gets the chunk's sum in slot c + k of
+// pose_partials (unique: a later chunk's first view is at least this chunk's last), which k_pose_reduce
+// sums over the view's chunks in order.
 //
 // Bound by the latency of its chain of loads (item -> record bits -> records) and by DRAM (16 aerial views
 // of 2M Gaussians, 7.4M live items: 1.7 GB at 4.2 TB/s, 55% of the issue slots). So: small blocks with one
 // barrier per chunk, four times as many as are resident (the multiprocessors that get the lighter chunks
 // take more blocks), the records of four pairs in flight, storage types and colour mode fixed at compile
-// time. 500 -> 407 us there, 8 views of 250k 80 -> 74, one of 100k 22 -> 20, one of 60k with third-degree
+// time. 500 -> 407 us there, 8 views of 500k 80 -> 74, one of 100k 22 -> 20, one of 60k with third-degree
 // harmonics 28 -> 23. Blocks of 256 threads 433, of 64 394 (but twice the sums for k_pose_reduce), only the
 // resident blocks 490; two pairs in flight and 5 blocks of 256 per SM 518; the parameters loaded before
 // the records 499 (spills).
@@ -167,13 +168,13 @@ __global__ void __launch_bounds__(kPoseBlock, SH ? 7 : 8) k_item_grads(Layout L,
     const Sum10 s = sum_pairs_warp(pg, pvalid, off, cnt, L.cap, valid);
     float pose[6] = {0, 0, 0, 0, 0, 0};
     if (valid) {
-    float p[3], ls[3], q[4];
+      float p[3], ls[3], q[4];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) p[j] = MF32 ? load_attr(G.means, 3 * g + j, GS_F32) : load_attr(G.means, 3 * g + j, G.means_dtype);
+      for (int j = 0; j < 3; ++j) p[j] = MF32 ? load_attr(G.means, 3 * g + j, GS_F32) : load_attr(G.means, 3 * g + j, G.means_dtype);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, DT);
+      for (int j = 0; j < 3; ++j) ls[j] = load_attr(G.log_scales, 3 * g + j, DT);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, DT);
+      for (int j = 0; j < 4; ++j) q[j] = load_attr(G.quats, 4 * g + j, DT);
       const float qlen = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
       const float iq = qlen > 0.0f ? 1.0f / qlen : 0.0f;
       const float w = q[0] * iq, x = q[1] * iq, y = q[2] * iq, z = q[3] * iq;

@@ -229,7 +229,8 @@ __device__ __forceinline__ TileCoord tile_coord(const Layout& L, int64_t tile_g)
 // one on most scenes from 3600 tiles on (loss-fused forward + backward, us at 2 / 4 pixels, 9 views of 640x480:
 // room 955 / 790, free 877 / 715), but where a few tiles have far longer lists than the others their two
 // warps set the time, on larger grids the longer the more Gaussians (aerial scene: 1200 tiles 338 / 430, 4032
-// 438 / 561, 10800 913 / 1066, 57600 4840 / 3840), and the host does not know the lists. The autotuner measures.
+// 438 / 561, 10800 913 / 1066, 14400 1273 / 1269, 21600 1849 / 1748, 28800 2467 / 2251, 57600 4840 / 3840), and the
+// host does not know the lists. The autotuner measures.
 // A caller who fixes only one of the two passes gets 2 for the other.
 int pick_px(int requested, int fallback) { return (requested == 1 || requested == 2 || requested == 4) ? requested : fallback; }
 int default_px(const Layout& L) {

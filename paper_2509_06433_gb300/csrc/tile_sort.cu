@@ -47,7 +47,7 @@ __device__ __forceinline__ uint32_t task_bound(const Layout& L, uint64_t pairs) 
 // One block per projection block: compacts its live items (in item order) and writes one record
 // (depth bits, slot, Gaussian id) per pair at the next free place of its tile's sub-list: the tile
 // scan has split every list between the projection blocks b with the same b % kTileSubLists. The
-// rate is set by the cursors' atomics, about one per 30 cycles on one address and fewer when the
+// rate is set by the cursors' atomics, about one warp's per 30 cycles on one address and fewer when the
 // cursors of neighbouring tiles share a 32-byte sector, so that the fullest tile decides: one sector
 // per cursor and four cursors per tile. The rows of a warp's items are numbered consecutively and
 // examined one per lane (row_span gives the same tiles as in the projection), then the pairs of those
