@@ -887,11 +887,16 @@ def roofline(stage, ms_list, counts, pairs, s, r, name):
                         f"{FLOP_BWD_EVAL:g} per backward evaluation x {counts['evals_bwd']}",
                 "peak_source": f"FP32 = {sms} SMs x 128 lanes x 2 x {mhz:.0f} MHz (max clock; nominal unit counts, "
                                f"{src} clock)"}
-    # HBM-bound stages: algorithmic bytes
-    passes = r.layout.sort_passes
+    # HBM-bound stages: the bytes of the form that runs, over the live items (those that emit pairs)
     N, K = s.N, s.K
-    bytes_ = {"project": N * 56 + K * N * (16 * 3 + 8) + N * 16,
-              "bin_sort": K * N * (4 * 16 + 24) + pairs * (12 + passes * 24 + 8),
+    mask = r.ws_view("live_mask", torch.int32, (K * N + 31) // 32).cpu().numpy().view(np.uint8)
+    live = int(np.unpackbits(mask).sum())
+    passes = r.layout.sort_passes
+    if r.layout.project_launches == 1:  # tile sort: staged records and lists in, one unsorted record per pair, lists out
+        bin_bytes = live * (4 + 48 + 12) + pairs * (16 + 16 + 12) + K * r.layout.tiles_x * r.layout.tiles_y * 8
+    else:  # radix sorts: 4 passes over the items' 8 bytes, their scan and table, `passes` over the pairs' 12
+        bin_bytes = live * (4 * 16 + 24) + pairs * (12 + passes * 24 + 8)
+    bytes_ = {"project": N * 56 + live * (16 * 3 + 8) + N * 16, "bin_sort": bin_bytes,
               "loss": K * s.H * s.W * 4 * (4 + 4 + 4),
               "project_bwd": N * 56 + pairs * 48 + N * 56}.get(stage, 0)
     hbm = float(peaks.get("hbm_gbs", 6800.0))
