@@ -472,9 +472,10 @@ __global__ void __launch_bounds__(kShortThreads) k_tile_sort(Layout L, uint8_t* 
 // written as one number, ((depth - least depth) << slot bits) | (slot - least slot). Either range loses 11
 // bits each time, so no list is cut more than seven times (32 and 30 bits). The record buffers are the 16
 // bytes per pair of pair_grads from byte 0 and from byte 16 capacity on; the third 16 bytes hold the slices
-// still to be cut. Projection and binning of 12,000 / 200,000 pairs of one tile, us: all depths equal 78 / 742
-// (932 / 18,311 when such slices went through a network of compare-exchanges in global memory), half of them
-// equal 110 / 1003 (484 / 8954), all different 82 / 784.
+// still to be cut. Projection and binning of 12,000 pairs of one tile, and of 200,000 by one block (the many of
+// run_tasks take 134 to 225), us: all depths equal 78 and 742 (932 and 18,311 when such slices went through a
+// network of compare-exchanges in global memory), half of them equal 110 and 1003 (484 and 8954), all different
+// 82 and 784.
 struct LongSmem {
   ListSmem<kLongShared> list;
   uint32_t slice[kLongSlices];
